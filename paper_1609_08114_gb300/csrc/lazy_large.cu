@@ -1,0 +1,18 @@
+// lazy_large.cu -- the pivots kept, FP32, the tableau kernel's arithmetic (m or n above 127).
+#include "simplex_lazy.cuh"
+
+namespace lpb {
+
+namespace {
+const LazyConfig kTable[] = {lazy_config<float, 4, 2, 4, true>(), lazy_config<float, 8, 2, 2, true>(), lazy_config<float, 8, 4, 1, true>()};
+}  // namespace
+
+cudaError_t lazy_occupancy_large(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay) {
+  return lazy_occ<float>(kTable, q, dtype, ctas, threads, lay);
+}
+
+cudaError_t launch_lazy_large(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s) {
+  return lazy_launch(kTable, p, lay, grid, s);
+}
+
+}  // namespace lpb

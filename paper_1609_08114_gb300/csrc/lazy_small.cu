@@ -1,0 +1,18 @@
+// lazy_small.cu -- the pivots kept, FP32, the register kernel's arithmetic (m, n <= 127).
+#include "simplex_lazy.cuh"
+
+namespace lpb {
+
+namespace {
+const LazyConfig kTable[] = {lazy_config<float, 1, 1, 16, false>(), lazy_config<float, 1, 2, 16, false>(), lazy_config<float, 2, 2, 8, false>()};
+}  // namespace
+
+cudaError_t lazy_occupancy_small(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay) {
+  return lazy_occ<float>(kTable, q, dtype, ctas, threads, lay);
+}
+
+cudaError_t launch_lazy_small(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s) {
+  return lazy_launch(kTable, p, lay, grid, s);
+}
+
+}  // namespace lpb

@@ -63,12 +63,16 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 enum ListKind { LIST_ALL = 0, LIST_CLASS = 1, LIST_DEFER = 2, LIST_RESOLVE = 3 };
 
+enum LazyKind { LAZY_NONE = 0, LAZY_SMALL = 1, LAZY_LARGE = 2, LAZY_FP64 = 3 };
+
 struct Pass {
   bool fp64 = false, gmem = false;
   int kcap = 0, mode = MODE_FP64, grid = 0, threads = 128;
   int reg = -1;              // >= 0: register-resident kernel configuration
   int pack = 0;              // > 0: several LPs per warp, this many lanes per LP
   bool warp = false;         // one warp per LP, the tableau in shared memory
+  int lazy = LAZY_NONE;      // the tableau kept as its pivots
+  LazyLayout lay = {};
   int list = LIST_ALL, cls = 0;
   int lim_m = 0, lim_n = 0;  // size bounds of the launch
   int group = 0;             // timing group: 0 first solve, 1 Phase-I pass, 2 FP64 re-solve
@@ -243,8 +247,58 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
   return rc <= 1;
 }
 
+// Gives a first pass to the kernel that keeps the pivots instead of a tableau
+// (simplex_lazy.cuh), with the arithmetic of the kernel that had the pass, so
+// the pivots are the same.  Every size up to 1024 under the largest-coefficient
+// rule, unless a kernel shape is asked for or several LPs share a warp: measured
+// faster at every size tried (type-1 LPs, ms per solve before and after):
+//   30,000 x 48 x 37, FP32 input   1.43 -> 0.28    50,000 x 64    1.46 -> 0.68
+//   50,000 x 100                   4.19 -> 2.11    2,000 x 300    6.0 -> 1.8-2.1
+//   20,000 x 100, FP64 tableau    12.42 -> 1.38
+// The random rule takes over three times the pivots (45.6 against 13.3 at
+// 100 x 100), which favours a full update; it stays with the kernels that do one.
+// History entries in shared memory: about what a type-1 LP's pivots need (13 at
+// 100 x 100, 33 at 300 x 300); more of them cost LPs in flight (50,000 x 100:
+// 2.38 ms with 8, 2.18 with 12, 2.12 with 16, 2.18 with 20; 2,000 x 300: 2.37
+// with 16, 2.06 with 30, 3.16 with 48).  FP64 entries are twice as large and its
+// chains are bound by the FP64 pipe, so fewer pay (20,000 x 100: 1.38 with 8,
+// 1.53 with 12).  At most kmax pivots: an LP beyond it starts again in the
+// tableau kernel, so it lies above what LPs with a bound on every variable take
+// (200 x 100, 64 pivots on average, 100 at most: 10,000 in 9.5 ms with none
+// handed on, 16 ms with 45% handed on, 17.5 ms all by the tableau kernel).
+void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, Pass *p) {
+  if (o->kernel != LPB_KERNEL_AUTO || o->threads != 0 || o->reg_warps != 0) return;
+  if (o->pivot_rule != LPB_PIVOT_LPC || p->pack > 0) return;
+  const int kind = p->fp64 ? LAZY_FP64 : (p->warp || p->reg >= 0) ? LAZY_SMALL : LAZY_LARGE;
+  const int eb = p->fp64 ? 8 : 4;
+  LazyShape q{};
+  q.max_m = p->lim_m;
+  q.max_n = p->lim_n;
+  const int mn = q.max_m < q.max_n ? q.max_m : q.max_n;
+  q.kmax = (64 + mn / 2 + 3) & ~3;
+  q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : kind == LAZY_SMALL ? 6 + mn / 10 : 8 + mn / 4;
+  const int most = 72 * 1024 / ((q.max_m + q.max_n) * eb);      // a third of an SM's shared memory
+  if (q.ks > most) q.ks = most > 1 ? most : 1;
+  int occ = 0, threads = 0;
+  LazyLayout lay{};
+  const cudaError_t ce = kind == LAZY_FP64 ? lazy_occupancy_fp64(q, b->dtype, &occ, &threads, &lay)
+                       : kind == LAZY_SMALL ? lazy_occupancy_small(q, b->dtype, &occ, &threads, &lay)
+                                            : lazy_occupancy_large(q, b->dtype, &occ, &threads, &lay);
+  if (ce != cudaSuccess) cudaGetLastError();
+  if (ce != cudaSuccess || occ < 1) return;                      // too large: the pass stays as it is
+  lay.tab = p->warp ? warp_tab_bytes(q.max_m, q.max_n) : 0;
+  p->lazy = kind;
+  p->lay = lay;
+  p->threads = threads;
+  p->smem = size_t(lay.bytes);
+  p->slot_bytes = (size_t(q.kmax - q.ks) * lay.hs * eb + 127) & ~size_t(127);
+  p->gmem = true;
+  p->grid = occ * d.sms;
+  if (p->grid > b->count) p->grid = b->count > 0 ? b->count : 1;
+}
+
 lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, bool basis_given,
-                  Plan *pl) {
+                  Plan *pl, bool lazy = true) {
   if (!b || !o) return LPB_EINVAL;
   if (b->count < 0) return LPB_EINVAL;
   if (b->max_m < 1 || b->max_n < 1 || b->max_m > kMaxDim || b->max_n > kMaxDim) return LPB_EUNSUPPORTED;
@@ -375,6 +429,8 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
     p.lim_n = b->max_n;
     np = 1;
   }
+  if (lazy)
+    for (int i = 0; i < np; ++i) lazy_pass(d, b, o, &pl->pass[i]);
   {                                // LPs that need more artificial columns (Phase I)
     Pass &p = pl->pass[np];
     if ((e = make_pass(d, b, &og, !fp32, b->max_m, mode, &p)) != LPB_OK) return e;
@@ -446,9 +502,9 @@ DeviceInfo device_info(const lpb_handle *h) { return DeviceInfo{h->sms, h->smem_
 namespace lpb {
 
 lpb_err solve_workspace_bytes(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
-                              bool basis_given, size_t *bytes) {
+                              bool basis_given, size_t *bytes, bool least) {
   Plan pl;
-  const lpb_err e = make_plan(d, b, o, basis_given, &pl);
+  const lpb_err e = make_plan(d, b, o, basis_given, &pl, !least);
   if (e != LPB_OK) return e;
   *bytes = pl.total;
   return LPB_OK;
@@ -462,6 +518,10 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
   Plan pl;
   lpb_err e = make_plan(d, b, o, r->basis != nullptr, &pl);
   if (e != LPB_OK) return e;
+  if (ws_bytes < pl.total) {       // less scratch than asked for: the kernels that need no history slots
+    pl = Plan();
+    if ((e = make_plan(d, b, o, r->basis != nullptr, &pl, false)) != LPB_OK) return e;
+  }
   if (ws_bytes < pl.total || (pl.total > 0 && !ws)) return LPB_ENOMEM;
   if (reinterpret_cast<uintptr_t>(ws) & 255) return LPB_EINVAL;
   unsigned char *w = static_cast<unsigned char *>(ws);
@@ -523,7 +583,10 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
         p.eps_d = pl.eps_d64;
         break;
     }
-    const cudaError_t ce = ps.pack > 0 ? launch_pack(p, ps.pack, ps.grid, s)
+    const cudaError_t ce = ps.lazy == LAZY_SMALL ? launch_lazy_small(p, ps.lay, ps.grid, s)
+                         : ps.lazy == LAZY_LARGE ? launch_lazy_large(p, ps.lay, ps.grid, s)
+                         : ps.lazy == LAZY_FP64 ? launch_lazy_fp64(p, ps.lay, ps.grid, s)
+                         : ps.pack > 0 ? launch_pack(p, ps.pack, ps.grid, s)
                          : ps.warp ? launch_warp(p, ps.grid, ps.threads, ps.smem, s)
                          : ps.reg >= 0 ? launch_reg(p, ps.reg, ps.grid, ps.smem, s)
                                        : launch_tableau(p, ps.fp64, ps.grid, ps.threads, ps.smem, s);
@@ -1179,6 +1242,7 @@ lpb_err lpb_autotune(lpb_handle *h, const lpb_batch *b, const lpb_options *o, co
   struct Cand { int kernel, threads, reg_warps; };
   const bool fp32 = o->prec != LPB_FP64;
   const Cand cands[] = {
+      {LPB_KERNEL_AUTO, 0, 0},
       {LPB_KERNEL_AUTO, 0, fp32 ? 8 : 0}, {LPB_KERNEL_AUTO, 0, fp32 ? 4 : 0}, {LPB_KERNEL_AUTO, 0, fp32 ? 1 : 0},
       {LPB_KERNEL_AUTO, 256, fp32 ? 8 : 0},
       {LPB_KERNEL_AUTO, 512, fp32 ? 8 : 0}, {LPB_KERNEL_AUTO, 1024, fp32 ? 8 : 0}, {LPB_KERNEL_SMEM, 0, 0},

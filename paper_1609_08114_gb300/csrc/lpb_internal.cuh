@@ -428,6 +428,34 @@ cudaError_t launch_pack(const TableauParams &p, int lanes, int grid, cudaStream_
 bool warp_fits(int max_m, int max_n);
 cudaError_t warp_occupancy(int max_m, int max_n, int *ctas, int *threads, size_t *smem);
 cudaError_t launch_warp(const TableauParams &p, int grid, int threads, size_t smem, cudaStream_t s);
+// Basic structurals the warp kernel's refinement takes at most, and the bytes
+// of its tableau region, which the refinement's operands must fit: LPs beyond
+// either go to the FP64 re-solve.  The lazy kernel keeps that limit where it has
+// the warp kernel's pass, so that the same LPs are re-solved (a re-solve counts
+// its own pivots and orders the basis its own way).
+constexpr int kWarpRefK = 24;
+int warp_tab_bytes(int max_m, int max_n);
+// The pivots kept instead of a tableau (simplex_lazy.cuh): shared-memory layout
+// of a launch, occupancy (0 CTAs: too large) and launch.  small: FP32, m and n up
+// to 127, the register kernel's arithmetic; large: FP32, the tableau kernel's;
+// fp64: FP64.
+struct LazyShape {
+  int max_m, max_n;
+  int ks, kmax;                // history entries in shared memory; pivots at most
+};
+struct LazyLayout {
+  int hs;                      // elements of a history entry
+  int ks, kmax;
+  int tab;                     // > 0: the warp kernel's limit on basic structurals, from these bytes
+  int hist, rp, at, xq, dv, off, kr, flag, red;   // byte offsets
+  int bytes;
+};
+cudaError_t lazy_occupancy_small(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay);
+cudaError_t lazy_occupancy_large(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay);
+cudaError_t lazy_occupancy_fp64(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay);
+cudaError_t launch_lazy_small(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
+cudaError_t launch_lazy_large(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
+cudaError_t launch_lazy_fp64(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
 size_t hyperbox_smem_bytes(int n, int elem_bytes, bool shared_box);
 cudaError_t launch_hyperbox(const HyperboxParams &p, uint32_t *err, cudaStream_t s);
 // Backward kernel (backward.cu).
@@ -445,9 +473,11 @@ struct DeviceInfo {
 
 constexpr int kCounters = 8;   // device int32 work queues and list lengths of one solve
 
-// Workspace bytes of a solve (`basis_given`: the caller passes a basis array).
+// Workspace bytes of a solve (`basis_given`: the caller passes a basis array);
+// `least`: of the plan without history slots, which run_solve takes when the
+// workspace holds no more.
 lpb_err solve_workspace_bytes(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
-                              bool basis_given, size_t *bytes);
+                              bool basis_given, size_t *bytes, bool least = false);
 // Zero `ctr` (kCounters device ints) and launch every pass of a solve on `s`,
 // with scratch from `ws`.  prof_ev (3 pairs) / prof_ran (3 flags) may be null.
 // lp_base: batch index of the batch's LP 0 (a chunk of a larger batch), which

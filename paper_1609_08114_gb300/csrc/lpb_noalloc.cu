@@ -78,7 +78,7 @@ extern "C" lpb_err lpb_solve_noalloc(const lpb_batch *b, const lpb_options *o, c
   lpb_err e = scratch_for_current_device(&s);
   if (e != LPB_OK) return e;
   size_t need = 0;
-  e = lpb::solve_workspace_bytes(s->info, b, o, r->basis != nullptr, &need);
+  e = lpb::solve_workspace_bytes(s->info, b, o, r->basis != nullptr, &need, true);
   if (e != LPB_OK) return e;
   if (need > kNoAllocBytes - kHeaderBytes) return LPB_ENOMEM;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -1003,6 +1003,8 @@ bool warp_fits(int max_m, int max_n) {
   return max_m >= 1 && max_n >= 1 && max_m <= kWarpMaxDim && max_n <= kWarpMaxDim;
 }
 
+int warp_tab_bytes(int max_m, int max_n) { return warp_layout(max_m, max_n).tab; }
+
 // Warps (LPs) per CTA and shared memory of the warp kernel for LPs up to
 // max_m x max_n: as many warps as the SM's shared memory holds regions, at most
 // eight; CTAs per SM from the occupancy calculator.
