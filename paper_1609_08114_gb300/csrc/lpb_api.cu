@@ -71,8 +71,9 @@ struct Pass {
   int reg = -1;              // >= 0: register-resident kernel configuration
   int pack = 0;              // > 0: several LPs per warp, this many lanes per LP
   bool warp = false;         // one warp per LP, the tableau in shared memory
-  int lazy = LAZY_NONE;      // the tableau kept as its pivots
+  int lazy = LAZY_NONE;      // the pivots kept instead of a tableau
   LazyLayout lay = {};
+  bool defer = false;        // tableau kernel with deferred updates
   int list = LIST_ALL, cls = 0;
   int lim_m = 0, lim_n = 0;  // size bounds of the launch
   int group = 0;             // timing group: 0 first solve, 1 Phase-I pass, 2 FP64 re-solve
@@ -112,18 +113,35 @@ int auto_threads(int eb, int rows, int cols, size_t smem) {
   return t;
 }
 
+// Whether a pass of the tableau kernel defers its updates (run_phase_deferred):
+// FP32, the largest-coefficient rule, no shape asked for, arrays of the waiting
+// pivots within 64 KB of shared memory, and a tableau of at least 1,700 entries
+// once Phase I has added half of the rows as columns, in at least 28 rows --
+// below that a full update costs less than the chains (14 x 190 0.593 and 0.623
+// ms per 2,000 LPs; two-phase LPs, ms of the Phase-I pass without and
+// with, 6,000 LPs: 24 x 24 1.08 and 1.23, 30 x 40 1.61 and 1.54, 60 x 20 2.81 and
+// 2.30, 60 x 60 6.2 and 3.7, 80 x 80 16.2 and 9.8; 4,000 x 200 x 200 193 and 71).
+// FP64 does not gain: its update is bound by the FP64 pipe, not by the sweeps.
+bool tableau_defers(const lpb_batch *b, const lpb_options *o, bool fp64, int kcap) {
+  if (fp64 || o->kernel != LPB_KERNEL_AUTO || o->threads != 0 || o->pivot_rule != LPB_PIVOT_LPC) return false;
+  if (tableau_fixed_bytes(4, b->max_m, b->max_n, kcap, false, true) -
+      tableau_fixed_bytes(4, b->max_m, b->max_n, kcap, false, false) > 64 * 1024) return false;
+  return b->max_m >= 28 && (b->max_m + 2) * (b->max_n + b->max_m / 2) >= 1700;
+}
+
 // A pass of the tableau kernel.  Its tableau rows go to shared memory as far
 // as they fit (all of them for the SMEM class), the rest to a per-CTA slot of
 // the workspace, sized so that the slots of all CTAs stay within about 3/4 of
 // L2; LPB_KERNEL_GMEM puts every row in the slot.
 lpb_err make_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, bool fp64, int kcap,
-                  int mode, Pass *p) {
+                  int mode, bool plain, Pass *p) {
   const int eb = fp64 ? 8 : 4;
   const bool refine = (mode == MODE_FP32_REFINE) && !fp64;
   p->fp64 = fp64;
   p->kcap = kcap;
   p->mode = mode;
-  const size_t fixed = tableau_fixed_bytes(eb, b->max_m, b->max_n, kcap, refine);
+  const bool defer = !plain && tableau_defers(b, o, fp64, kcap);
+  const size_t fixed = tableau_fixed_bytes(eb, b->max_m, b->max_n, kcap, refine, defer);
   const size_t rowb = tableau_row_bytes(eb, b->max_n, kcap);
   const size_t rows = size_t(b->max_m) + 2;
   // Leave room for the kernel's static shared memory.
@@ -154,11 +172,14 @@ lpb_err make_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
   p->gmem = p->slot_bytes > 0;
   p->smem = fixed + p->tab_smem;
   if (p->smem < 16) p->smem = 16;
+  p->defer = defer;
   p->threads = o->threads > 0 ? o->threads
+             // (128 registers per thread keep a lane's waiting pivot rows: 256 threads, two CTAs per SM)
+             : defer ? (b->max_m * b->max_n >= 6000 ? 256 : 128)
              : auto_threads_override ? auto_threads_override : auto_threads(eb, int(rows), int(rowb / eb), p->smem);
   if (p->threads < 32 || p->threads > 1024 || (p->threads & 31)) return LPB_EINVAL;
   int occ = 0;
-  if (tableau_max_ctas_per_sm(eb, p->threads, p->smem, &occ) != cudaSuccess) return LPB_ECUDA;
+  if (tableau_max_ctas_per_sm(eb, p->threads, p->smem, defer, &occ) != cudaSuccess) return LPB_ECUDA;
   if (occ < 1) return LPB_EUNSUPPORTED;
   p->grid = occ * d.sms;
   if (p->gmem) {
@@ -297,8 +318,10 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, Pa
   if (p->grid > b->count) p->grid = b->count > 0 ? b->count : 1;
 }
 
+// `plain`: full updates after every pivot in every pass (no history slots, more
+// rows in shared memory).
 lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, bool basis_given,
-                  Plan *pl, bool lazy = true) {
+                  Plan *pl, bool plain = false) {
   if (!b || !o) return LPB_EINVAL;
   if (b->count < 0) return LPB_EINVAL;
   if (b->max_m < 1 || b->max_n < 1 || b->max_m > kMaxDim || b->max_n > kMaxDim) return LPB_EUNSUPPORTED;
@@ -402,7 +425,7 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
       pl->nclass = nreg + (covered ? 0 : 1);
       if (!covered) {              // the largest LPs first: the tableau kernel's class
         Pass &p = pl->pass[np];
-        if ((e = make_pass(d, b, &og, false, 0, mode, &p)) != LPB_OK) return e;
+        if ((e = make_pass(d, b, &og, false, 0, mode, plain, &p)) != LPB_OK) return e;
         p.list = LIST_CLASS;
         p.cls = nreg;
         p.lim_m = b->max_m;
@@ -421,7 +444,7 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
     if (o->kernel == LPB_KERNEL_REG && reg < 0) return LPB_EUNSUPPORTED;
     if (reg >= 0) {
       if ((e = reg_pass(d, b, reg, b->max_m, b->max_n, mode, o->pivot_rule, &p)) != LPB_OK) return e;
-    } else if ((e = make_pass(d, b, &og, !fp32, 0, mode, &p)) != LPB_OK) {
+    } else if ((e = make_pass(d, b, &og, !fp32, 0, mode, plain, &p)) != LPB_OK) {
       return e;
     }
     p.list = LIST_ALL;
@@ -429,11 +452,11 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
     p.lim_n = b->max_n;
     np = 1;
   }
-  if (lazy)
+  if (!plain)
     for (int i = 0; i < np; ++i) lazy_pass(d, b, o, &pl->pass[i]);
   {                                // LPs that need more artificial columns (Phase I)
     Pass &p = pl->pass[np];
-    if ((e = make_pass(d, b, &og, !fp32, b->max_m, mode, &p)) != LPB_OK) return e;
+    if ((e = make_pass(d, b, &og, !fp32, b->max_m, mode, plain, &p)) != LPB_OK) return e;
     p.list = LIST_DEFER;
     p.group = 1;
     p.lim_m = b->max_m;
@@ -443,7 +466,7 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
   pl->resolve = o->prec == LPB_FP32_REFINE;
   if (pl->resolve) {               // FP64 re-solve of the LPs that failed the FP32 certificate
     Pass &p = pl->pass[np];
-    if ((e = make_pass(d, b, &og, true, b->max_m, MODE_FP64, &p)) != LPB_OK) return e;
+    if ((e = make_pass(d, b, &og, true, b->max_m, MODE_FP64, plain, &p)) != LPB_OK) return e;
     p.list = LIST_RESOLVE;
     p.group = 2;
     p.lim_m = b->max_m;
@@ -504,7 +527,7 @@ namespace lpb {
 lpb_err solve_workspace_bytes(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
                               bool basis_given, size_t *bytes, bool least) {
   Plan pl;
-  const lpb_err e = make_plan(d, b, o, basis_given, &pl, !least);
+  const lpb_err e = make_plan(d, b, o, basis_given, &pl, least);
   if (e != LPB_OK) return e;
   *bytes = pl.total;
   return LPB_OK;
@@ -518,9 +541,9 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
   Plan pl;
   lpb_err e = make_plan(d, b, o, r->basis != nullptr, &pl);
   if (e != LPB_OK) return e;
-  if (ws_bytes < pl.total) {       // less scratch than asked for: the kernels that need no history slots
+  if (ws_bytes < pl.total) {       // less scratch than asked for: full updates, which need less
     pl = Plan();
-    if ((e = make_plan(d, b, o, r->basis != nullptr, &pl, false)) != LPB_OK) return e;
+    if ((e = make_plan(d, b, o, r->basis != nullptr, &pl, true)) != LPB_OK) return e;
   }
   if (ws_bytes < pl.total || (pl.total > 0 && !ws)) return LPB_ENOMEM;
   if (reinterpret_cast<uintptr_t>(ws) & 255) return LPB_EINVAL;
@@ -589,7 +612,7 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
                          : ps.pack > 0 ? launch_pack(p, ps.pack, ps.grid, s)
                          : ps.warp ? launch_warp(p, ps.grid, ps.threads, ps.smem, s)
                          : ps.reg >= 0 ? launch_reg(p, ps.reg, ps.grid, ps.smem, s)
-                                       : launch_tableau(p, ps.fp64, ps.grid, ps.threads, ps.smem, s);
+                                       : launch_tableau(p, ps.fp64, ps.defer, ps.grid, ps.threads, ps.smem, s);
     if (ce != cudaSuccess) return LPB_ECUDA;
     if (kernels) *kernels += 1;
   }

@@ -402,10 +402,10 @@ struct HyperboxParams {
 // kcap negated rows.  A launch holds `tab_smem` bytes of rows in shared
 // memory after those buffers and the rest of each tableau in a slot of
 // `slot_bytes` per CTA.
-size_t tableau_fixed_bytes(int elem_bytes, int max_m, int max_n, int kcap, bool refine);
+size_t tableau_fixed_bytes(int elem_bytes, int max_m, int max_n, int kcap, bool refine, bool defer);
 size_t tableau_row_bytes(int elem_bytes, int max_n, int kcap);
-cudaError_t tableau_max_ctas_per_sm(int elem_bytes, int threads, size_t smem, int *ctas);
-cudaError_t launch_tableau(const TableauParams &p, bool fp64, int grid, int threads, size_t smem, cudaStream_t s);
+cudaError_t tableau_max_ctas_per_sm(int elem_bytes, int threads, size_t smem, bool defer, int *ctas);
+cudaError_t launch_tableau(const TableauParams &p, bool fp64, bool defer, int grid, int threads, size_t smem, cudaStream_t s);
 // Register-resident FP32 kernel (simplex_reg.cu): configuration index for
 // (max_m, max_n) or -1, its occupancy, and its launch.  It defers to the
 // defer list every LP it does not take (Phase I, sizes, non-finite data).
@@ -474,7 +474,7 @@ struct DeviceInfo {
 constexpr int kCounters = 8;   // device int32 work queues and list lengths of one solve
 
 // Workspace bytes of a solve (`basis_given`: the caller passes a basis array);
-// `least`: of the plan without history slots, which run_solve takes when the
+// `least`: of the plan with full updates, which run_solve takes when the
 // workspace holds no more.
 lpb_err solve_workspace_bytes(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
                               bool basis_given, size_t *bytes, bool least = false);

@@ -96,9 +96,11 @@ __device__ __forceinline__ T a_in(const void *A, int i) {
 }
 
 // Largest magnitude image (FP64: the high word, FP32: the word) of the LP's
-// `cnt` entries of A, by 16-byte loads, kU in flight per thread.
-template <bool F64, int NT>
-__device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid) {
+// `cnt` entries of A, by 16-byte loads, kU in flight per thread.  `stop`, asked
+// once while the first are on their way, may end it (an LP that goes elsewhere
+// anyway is not read through).
+template <bool F64, int NT, typename F>
+__device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid, F &&stop) {
   constexpr int ES = F64 ? 8 : 4, PER = 16 / ES, kU = 8;
   const unsigned char *p = static_cast<const unsigned char *>(A);
   int head = int((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / ES;
@@ -108,24 +110,37 @@ __device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid) {
     const unsigned u = F64 ? __ldg(reinterpret_cast<const uint2 *>(p) + i).y : __ldg(reinterpret_cast<const unsigned *>(p) + i);
     amax = max(amax, u & 0x7fffffffu);
   };
-  if (tid < head) one(tid);
   const int nv = (cnt - head) / PER;
   const uint4 *v4 = reinterpret_cast<const uint4 *>(p + size_t(head) * ES);
   auto fold = [&](const uint4 &v) {
     if (!F64) amax = max(amax, max(v.x & 0x7fffffffu, v.z & 0x7fffffffu));
     amax = max(amax, max(v.y & 0x7fffffffu, v.w & 0x7fffffffu));
   };
-  int k = tid;
+  uint4 v[kU];
+  if (nv > 0) {                    // the first loads; past the end the last vector again
+#pragma unroll
+    for (int u = 0; u < kU; ++u) v[u] = __ldg(v4 + min(tid + u * NT, nv - 1));
+  }
+  if (stop()) return 0u;
+  if (nv > 0) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) fold(v[u]);
+  }
+  int k = tid + kU * NT;
 #pragma unroll 1
   for (; k + (kU - 1) * NT < nv; k += kU * NT) {
-    uint4 v[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) v[u] = __ldg(v4 + k + u * NT);
 #pragma unroll
     for (int u = 0; u < kU; ++u) fold(v[u]);
   }
-#pragma unroll 1
-  for (; k < nv; k += NT) fold(__ldg(v4 + k));
+  if (k - tid < nv) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) v[u] = __ldg(v4 + min(k + u * NT, nv - 1));
+#pragma unroll
+    for (int u = 0; u < kU; ++u) fold(v[u]);
+  }
+  if (tid < head) one(tid);
   const int done = head + nv * PER;
   if (done + tid < cnt) one(done + tid);      // fewer than PER entries are left
   return amax;
@@ -257,7 +272,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     int rst[R], cst[R];            // last pivot on each row and column, -1: none
     int ic[R], jc[R];              // own rows and columns; past the end the last one (read, never used)
     bool in_m[R], in_n[R];
-    if (fits) {
+    if (fits) {                    // (the same in every thread)
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int i = tid + NT * r;
@@ -291,10 +306,10 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
           obj[r] = -d2f_tile(c, bad);
         }
       }
-      const unsigned amax = scan_a<F64, NT>(A, m * n, tid);
+      bad |= int(bm >= kInf) | int(cm >= kInf);
+      const unsigned amax = scan_a<F64, NT>(A, m * n, tid, [&]() { return any(bad); });
       // Not finite, or (FP32) so large that rounding could leave the float range.
       bad |= int(amax >= (F64 ? (kD ? 0x7ff00000u : 0x47efffffu) : 0x7f800000u));
-      bad |= int(bm >= kInf) | int(cm >= kInf);
     }
     bm = warp_max_u64(bm);
     cm = warp_max_u64(cm);

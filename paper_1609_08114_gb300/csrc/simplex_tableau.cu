@@ -13,6 +13,8 @@
 //    (none for most LPs) in a per-CTA workspace slot that stays in L2.  Rows
 //    have an odd leading dimension, so the column reads of Step 2 are free of
 //    bank conflicts.
+//  * Updates: full after every pivot as below, or deferred (FP32 under the
+//    largest-coefficient rule from a few thousand entries on: run_phase_deferred).
 //  * Work split: warp w owns a contiguous block of rows; lanes own columns.
 //    One pivot takes two block barriers.  Before the first, every warp runs
 //    Step 2 on its own rows (a warp arg-min, one slot per warp) and the
@@ -41,9 +43,28 @@ namespace lpb {
 namespace {
 
 constexpr int kMaxThreads = 1024;
+// Deferred updates (run_phase_deferred): threads per CTA at most and CTAs per SM
+// (128 registers per thread: 64 hold a lane's part of the waiting pivot rows in
+// the sweep), pivots that wait at most, the row stride of their multipliers
+// (16-byte rows without bank conflicts), rows in flight per warp in the sweep.
+// Measured on 4,000 two-phase LPs of 200 x 200 (ms of the Phase-I pass): 71; 8
+// pivots with three or four CTAs 118 (spills), 16 with three 146, 32 with two
+// 153, the next rows loaded while these are computed 73-74.
+constexpr int kDefThreads = 256;
+constexpr int kDefCtas = 2;
+constexpr int kDefer = 16;
+constexpr int kDeferLd = kDefer + 4;
+constexpr int kFlushRows = 4;
+
+// A warp's candidate column or row: value image and key, and two values of it.
+struct __align__(16) PivotRec {
+  unsigned o, key;
+  float a, b;
+};
 
 struct Layout {
-  size_t tab, colb, rowb, gam, basic, nonb, redv, redk, rcp, redf, sel, ins, wl, xb, rr, yv, rho, sb, ns, sp, dj, jq, kq, total;
+  size_t tab, colb, rowb, gam, basic, nonb, redv, redk, rcp, redf, sel, ins, wl, xb, rr, yv, rho, sb, ns, sp, dj, jq, kq;
+  size_t df, dp, rhs, obj, rec, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -56,7 +77,7 @@ __host__ __device__ inline int tab_ld(int n, int k, int eb) {
 }
 
 // Dynamic shared memory: `tab` bytes of tableau rows, then the buffers.
-__host__ __device__ inline Layout make_layout(int eb, size_t tab, int max_m, int max_n, int kcap, bool refine) {
+__host__ __device__ inline Layout make_layout(int eb, size_t tab, int max_m, int max_n, int kcap, bool refine, bool defer) {
   Layout L{};
   const size_t ld = size_t(tab_ld(max_n, kcap, eb));
   const size_t rows = size_t(max_m) + 2;
@@ -86,6 +107,13 @@ __host__ __device__ inline Layout make_layout(int eb, size_t tab, int max_m, int
     L.jq = o;  o = align16(o + size_t(max_m) * 4);
     L.kq = o;  o = align16(o + size_t(max_m) * 4);
   }
+  if (defer) {
+    L.df = o;  o = align16(o + rows * kDeferLd * 4);
+    L.dp = o;  o = align16(o + ld * kDefer * 4);
+    L.rhs = o; o = align16(o + rows * 4);
+    L.obj = o; o = align16(o + ld * 4);
+    L.rec = o; o = align16(o + 2 * (kDefThreads / 32) * sizeof(PivotRec));
+  }
   L.total = o;
   return L;
 }
@@ -111,6 +139,10 @@ struct Tab {
   unsigned char *ins;
   int *wl;        // warm start: columns whose variable enters
   int m, n, k, nc, ld;   // nc = n + k non-RHS columns; column nc is the RHS
+  // Deferred updates: multipliers by row and pivot rows of the waiting pivots,
+  // the right-hand side and the objective row as they are now.
+  float *df, *dp, *rhsv, *objv;
+  PivotRec *rec;
   int nm;                // variables >= nm are artificial
   __device__ __forceinline__ T *row(int i) const {
     return i < rs ? ts + size_t(i) * ld : tg + size_t(i - rs) * ld;
@@ -582,6 +614,265 @@ __device__ __forceinline__ int run_phase(Tab<T> &S_, int orow, int rows, int pha
   }
 }
 
+// All waiting pivots into the tableau's rows (all but `orow`, whose multipliers
+// are zero): a lane keeps its 16-byte vector of every waiting pivot row in
+// registers while the warp's rows stream past, four in flight.
+__device__ __forceinline__ void flush_deferred(const Tab<float> &S_, int rows) {
+  const Tab<float> S = S_;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int nv = (S.nc + 3) >> 2;
+  for (int v0 = lane; v0 < nv; v0 += 32) {
+    float4 p[kDefer];
+#pragma unroll
+    for (int s = 0; s < kDefer; ++s) p[s] = reinterpret_cast<const float4 *>(S.dp + s * S.ld)[v0];
+    auto load = [&](float4 (&x)[kFlushRows], int i0) {
+#pragma unroll
+      for (int u = 0; u < kFlushRows; ++u)
+        x[u] = reinterpret_cast<const float4 *>(S.row(min(i0 + u * nw, rows - 1)))[v0];
+    };
+    auto apply = [&](float4 (&x)[kFlushRows], int i0) {
+#pragma unroll
+      for (int u = 0; u < kFlushRows; ++u) {
+        const int i = i0 + u * nw;
+        if (i >= rows) break;
+        const float4 *f = reinterpret_cast<const float4 *>(S.df + i * kDeferLd);
+#pragma unroll
+        for (int s = 0; s < kDefer; s += 4) {
+          const float4 g = f[s / 4];
+          x[u] = upd_vec(x[u], p[s], -g.x);
+          x[u] = upd_vec(x[u], p[s + 1], -g.y);
+          x[u] = upd_vec(x[u], p[s + 2], -g.z);
+          x[u] = upd_vec(x[u], p[s + 3], -g.w);
+        }
+        reinterpret_cast<float4 *>(S.row(i))[v0] = x[u];
+      }
+    };
+    float4 x[kFlushRows];
+#pragma unroll 1
+    for (int i0 = w; i0 < rows; i0 += kFlushRows * nw) {
+      load(x, i0);
+      apply(x, i0);
+    }
+  }
+}
+
+// run_phase for FP32 under the largest-coefficient rule with the rank-1 updates
+// deferred.  With f_s the multipliers t_ie / p and p_s the (unscaled) pivot row
+// of pivot s, an entry as it is now is its stored value with x <- fma(-f_s[i],
+// p_s[j], x) run over the waiting pivots: the full update's operations in its
+// order, so every choice and every value is the same.  A pivot runs this for one
+// column and one row; the right-hand side and the objective row are kept
+// current in shared memory.  After it, row l and column e are stored as they
+// are now and their waiting multipliers set to zero, so that the chain skips
+// what they contain.  When kDefer pivots wait, one sweep applies them all.
+// Two barriers per pivot, as before; the tableau, most of it in L2 for large
+// LPs, is read and written once per kDefer pivots instead of once per pivot
+// (4,000 two-phase LPs of 200 x 200: 193 -> 71 ms).  What bounds it now: per
+// pivot the round trips to L2 for the column's and the row's entries between
+// the two barriers (5 of 9 thousand cycles per CTA), and the sweep (2.3).
+__device__ __forceinline__ int run_phase_deferred(Tab<float> &S_, int orow, int rows, int phase, int &iters,
+                                                  int max_iter, float eps_p, float eps_d) {
+  Tab<float> S = S_;   // a register copy: stores through tableau pointers cannot alias it
+  constexpr unsigned kNone = 0xffffffffu;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
+  PivotRec *rec1 = S.rec, *rec2 = S.rec + kDefThreads / 32;
+  auto zero_waiting = [&]() {
+    for (int t = tid; t < rows * kDeferLd; t += nt) S.df[t] = 0.f;
+    for (int t = tid; t < S.ld * kDefer; t += nt) S.dp[t] = 0.f;
+  };
+  for (int i = tid; i < rows; i += nt) S.rhsv[i] = S.at(i, S.nc);
+  for (int j = tid; j < S.nc; j += nt) S.objv[j] = S.row(orow)[j];
+  zero_waiting();
+  __syncthreads();
+  int degenerate_run = 0, wait = 0, prev_l = -1, status = LPB_OPTIMAL;
+  bool bland = false;
+  // A thread's best candidate, then its warp's into rec[w].
+  auto offer = [&](PivotRec *rec, unsigned o, unsigned key, float a, float b) {
+    const unsigned mo = __reduce_min_sync(kFull, o);
+    const unsigned mk = __reduce_min_sync(kFull, o == mo ? key : kNone);
+    if (mo == kNone) {
+      if (lane == 0) rec[w] = PivotRec{kNone, kNone, 0.f, 0.f};
+    } else if (o == mo && key == mk) {
+      rec[w] = PivotRec{mo, mk, a, b};
+    }
+  };
+  auto best_of = [&](const PivotRec *rec) -> PivotRec {
+    const PivotRec r = rec[lane < nw ? lane : 0];
+    const unsigned mo = __reduce_min_sync(kFull, r.o);
+    const unsigned mk = __reduce_min_sync(kFull, r.o == mo ? r.key : kNone);
+    const int src = __ffs(__ballot_sync(kFull, r.o == mo && r.key == mk)) - 1;
+    return PivotRec{mo, mk, __shfl_sync(kFull, r.a, src), __shfl_sync(kFull, r.b, src)};
+  };
+  {                        // Step 1 of the first pivot
+    unsigned o = kNone, key = kNone;
+    float a = 0.f;
+    for (int j = tid; j < S.nc; j += nt) {
+      const int var = S.nonb[j];
+      const float rj = S.objv[j];
+      if (var >= S.nm || !(rj < -eps_d)) continue;
+      const unsigned oj = f2ord(rj), kj = unsigned((var << kIdxBits) | j);
+      if (oj < o || (oj == o && kj < key)) { o = oj; key = kj; a = rj; }
+    }
+    offer(rec1, o, key, a, 0.f);
+  }
+  __syncthreads();
+  PivotRec col = best_of(rec1);
+  for (;;) {
+    if (prev_l >= 0 && tid == prev_l % nt)      // row l is stored as it is now
+      for (int s = 0; s < kDefer; s += 4)
+        *reinterpret_cast<float4 *>(S.df + prev_l * kDeferLd + s) = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (col.o == kNone) break;
+    const int e = int(col.key) & kIdxMask;
+    // Column e and Step 2.
+    {
+      unsigned o = kNone, key = kNone;
+      float a = 0.f, b = 0.f;
+      for (int i = tid; i < rows; i += nt) {
+        if (i == orow) continue;
+        float x = S.at(i, e);
+        const float *pe = S.dp + e;
+        const float4 *f = reinterpret_cast<const float4 *>(S.df + i * kDeferLd);
+#pragma unroll
+        for (int s = 0; s < kDefer; s += 4)
+          if (s < wait) {
+            const float4 g = f[s / 4];
+            x = fmaf(-g.x, pe[s * S.ld], x);
+            x = fmaf(-g.y, pe[(s + 1) * S.ld], x);
+            x = fmaf(-g.z, pe[(s + 2) * S.ld], x);
+            x = fmaf(-g.w, pe[(s + 3) * S.ld], x);
+          }
+        S.colb[i] = x;
+        if (i < S.m && x > eps_p) {
+          const int bv = S.basic[i];
+          if (phase == 2 && bv >= S.nm) continue;
+          const float r = S.rhsv[i];
+          const unsigned oi = f2ord(r / x), ki = unsigned((bv << kIdxBits) | i);
+          if (oi < o || (oi == o && ki < key)) { o = oi; key = ki; a = x; b = r; }
+        }
+      }
+      offer(rec2, o, key, a, b);
+    }
+    __syncthreads();
+    const PivotRec piv = best_of(rec2);
+    if (piv.o == kNone) { status = phase == 2 ? LPB_UNBOUNDED : LPB_NUMERIC; break; }
+    if (iters >= max_iter) { status = LPB_ITER_LIMIT; break; }
+    const int l = int(piv.key) & kIdxMask, leave = int(piv.key >> kIdxBits);
+    const float rp = 1.f / piv.a, bl = piv.b, fm = col.a * rp;
+    // Degenerate pivots, before Step 1 of the next pivot asks for Bland's rule.
+    if (ord2f(piv.o) <= eps_p) {
+      if (++degenerate_run >= S.m + S.n) bland = true;
+    } else {
+      degenerate_run = 0;
+      bland = false;
+    }
+    // Row l, the objective row and Step 1 of the next pivot.
+    {
+      unsigned o = kNone, key = kNone;
+      float a = 0.f;
+      float *rl = S.row(l);
+      const float4 *f = reinterpret_cast<const float4 *>(S.df + l * kDeferLd);
+      for (int j = tid; j < S.nc; j += nt) {
+        float q = rl[j];
+        float *pj = S.dp + j;
+#pragma unroll
+        for (int s = 0; s < kDefer; s += 4)
+          if (s < wait) {
+            const float4 g = f[s / 4];
+            q = fmaf(-g.x, pj[s * S.ld], q);
+            q = fmaf(-g.y, pj[(s + 1) * S.ld], q);
+            q = fmaf(-g.z, pj[(s + 2) * S.ld], q);
+            q = fmaf(-g.w, pj[(s + 3) * S.ld], q);
+          }
+        float rj;
+        int var;
+        if (j == e) {
+          rj = -fm;
+          var = leave;
+          rl[j] = rp;
+          for (int s = 0; s < wait; ++s) pj[s * S.ld] = 0.f;   // column e is stored as it is now
+        } else {
+          rj = fmaf(-fm, q, S.objv[j]);
+          var = S.nonb[j];
+          rl[j] = q * rp;
+          pj[wait * S.ld] = q;
+        }
+        S.objv[j] = rj;
+        if (var >= S.nm || !(rj < -eps_d)) continue;
+        const unsigned oj = bland ? f2ord(0.f) : f2ord(rj), kj = unsigned((var << kIdxBits) | j);
+        if (oj < o || (oj == o && kj < key)) { o = oj; key = kj; a = rj; }
+      }
+      offer(rec1, o, key, a, 0.f);
+    }
+    // The right-hand side and column e.
+    for (int i = tid; i < rows; i += nt) {
+      if (i == orow) {
+        S.rhsv[i] = fmaf(-fm, bl, S.rhsv[i]);
+      } else if (i == l) {
+        S.rhsv[i] = bl * rp;
+      } else {
+        const float g = S.colb[i] * rp;
+        S.rhsv[i] = fmaf(-g, bl, S.rhsv[i]);
+        S.df[i * kDeferLd + wait] = g;
+        S.at(i, e) = -g;
+      }
+    }
+    if (tid == 0) {
+      S.basic[l] = int(col.key >> kIdxBits);
+      S.nonb[e] = leave;
+    }
+    prev_l = l;
+    ++iters;
+    ++wait;
+    __syncthreads();
+    col = best_of(rec1);
+    if (phase == 1 && leave >= S.nm) {
+      // The artificial's new column is dead: the last column moves into it.
+      const int last = S.nc - 1;
+      if (e != last) {
+        for (int i = tid; i < rows; i += nt) S.at(i, e) = S.at(i, last);
+        for (int s = tid; s < kDefer; s += nt) S.dp[s * S.ld + e] = S.dp[s * S.ld + last];
+      }
+      __syncthreads();     // (the last column is read)
+      for (int i = tid; i < rows; i += nt) S.at(i, last) = 0.f;
+      for (int s = tid; s < kDefer; s += nt) S.dp[s * S.ld + last] = 0.f;
+      if (tid == 0 && e != last) {
+        S.nonb[e] = S.nonb[last];
+        S.objv[e] = S.objv[last];
+      }
+      if (col.o != kNone && (int(col.key) & kIdxMask) == last) col.key = (col.key & ~unsigned(kIdxMask)) | unsigned(e);
+      S.nc = last;
+      __syncthreads();
+    }
+    if (wait == kDefer) {
+      if (tid == prev_l % nt)
+        for (int s = 0; s < kDefer; ++s) S.df[prev_l * kDeferLd + s] = 0.f;
+      prev_l = -1;
+      __syncthreads();
+      flush_deferred(S, rows);
+      __syncthreads();
+      zero_waiting();
+      wait = 0;
+      __syncthreads();
+    }
+  }
+  // The tableau as it is now: the waiting pivots, the objective row, the
+  // right-hand side, zeros in the padding columns.
+  __syncthreads();
+  if (wait > 0) {
+    flush_deferred(S, rows);
+    __syncthreads();
+  }
+  for (int j = tid; j < S.nc; j += nt) S.row(orow)[j] = S.objv[j];
+  for (int i = tid; i < rows; i += nt) {
+    float *r = S.row(i);
+    r[S.nc] = S.rhsv[i];
+    for (int j = S.nc + 1; j < S.ld && j < S.nc + 5; ++j) r[j] = 0.f;
+  }
+  __syncthreads();
+  S_.nc = S.nc;
+  return status;
+}
+
 // Largest |t_ij| over enterable columns of row i (ties: lowest column); -1 if
 // none exceeds `eps`.
 template <typename T>
@@ -1011,14 +1302,15 @@ __device__ __forceinline__ bool refine_and_verify(const Tab<float> &S_, const Ba
   return true;
 }
 
-// FUSE_SE: the FP32 steepest-edge instantiation (see run_phase).
-template <typename T, bool FUSE_SE>
-__global__ void __launch_bounds__(kMaxThreads) tableau_kernel(TableauParams P) {
+// FUSE_SE: the FP32 steepest-edge instantiation (see run_phase); DEF: FP32 with
+// deferred updates (run_phase_deferred).
+template <typename T, bool FUSE_SE, bool DEF>
+__global__ void __launch_bounds__(DEF ? kDefThreads : kMaxThreads, DEF ? kDefCtas : 1) tableau_kernel(TableauParams P) {
   constexpr bool kFuseSE = FUSE_SE;
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, nt = blockDim.x;
   const bool refine = (P.mode == MODE_FP32_REFINE) && sizeof(T) == 4;
-  const Layout L = make_layout(int(sizeof(T)), P.tab_smem, P.B.max_m, P.B.max_n, P.kcap, refine);
+  const Layout L = make_layout(int(sizeof(T)), P.tab_smem, P.B.max_m, P.B.max_n, P.kcap, refine, DEF);
   Tab<T> S;
   S.ts = reinterpret_cast<T *>(smem + L.tab);
   S.tg = P.slot_bytes ? reinterpret_cast<T *>(static_cast<unsigned char *>(P.slots) + size_t(blockIdx.x) * P.slot_bytes)
@@ -1035,6 +1327,18 @@ __global__ void __launch_bounds__(kMaxThreads) tableau_kernel(TableauParams P) {
   S.sel = reinterpret_cast<int *>(smem + L.sel);
   S.ins = smem + L.ins;
   S.wl = reinterpret_cast<int *>(smem + L.wl);
+  if constexpr (DEF) {
+    S.df = reinterpret_cast<float *>(smem + L.df);
+    S.dp = reinterpret_cast<float *>(smem + L.dp);
+    S.rhsv = reinterpret_cast<float *>(smem + L.rhs);
+    S.objv = reinterpret_cast<float *>(smem + L.obj);
+    S.rec = reinterpret_cast<PivotRec *>(smem + L.rec);
+  }
+  // Steps 1-3 on one objective row.
+  auto run = [&](int orow, int rows, int phase, int &iters_, int max_iter_, T ep, T ed, int lp_) -> int {
+    if constexpr (DEF) return run_phase_deferred(S, orow, rows, phase, iters_, max_iter_, ep, ed);
+    else return run_phase<T, kFuseSE>(S, orow, rows, phase, iters_, max_iter_, ep, ed, P.rule, P.seed, P.lp_base + lp_);
+  };
   __shared__ int s_item, s_k;
   __shared__ unsigned long long s_bmax, s_cmax;
   const T eps_p = T(P.eps_p), eps_d = T(P.eps_d);
@@ -1141,7 +1445,7 @@ __global__ void __launch_bounds__(kMaxThreads) tableau_kernel(TableauParams P) {
           const int jm = row_argmax_abs(S, m + 1, T(0), 0);
           if (jm >= 0) eps_d1 = eps_d * fmaxf(1.f, fabsf(S.at(m + 1, jm)));
         }
-        status = run_phase<T, kFuseSE>(S, m + 1, m + 2, 1, iters, max_iter, eps_p, eps_d1, P.rule, P.seed, P.lp_base + lp);
+        status = run(m + 1, m + 2, 1, iters, max_iter, eps_p, eps_d1, lp);
         if (status == LPB_OPTIMAL) {
           const double w = double(S.at(m + 1, S.nc));
           if (-w > ftol) {
@@ -1160,7 +1464,7 @@ __global__ void __launch_bounds__(kMaxThreads) tableau_kernel(TableauParams P) {
           }
         }
       }
-      if (status == LPB_OPTIMAL) status = run_phase<T, kFuseSE>(S, m, m + 1, 2, iters, max_iter, eps_p, eps_d, P.rule, P.seed, P.lp_base + lp);
+      if (status == LPB_OPTIMAL) status = run(m, m + 1, 2, iters, max_iter, eps_p, eps_d, lp);
     }
     if constexpr (sizeof(T) == 4) if (P.mode == MODE_FP32_REFINE) {
       bool done = false;
@@ -1190,35 +1494,32 @@ __global__ void __launch_bounds__(kMaxThreads) tableau_kernel(TableauParams P) {
 
 }  // namespace
 
-size_t tableau_fixed_bytes(int eb, int max_m, int max_n, int kcap, bool refine) {
-  return make_layout(eb, 0, max_m, max_n, kcap, refine).total;
+size_t tableau_fixed_bytes(int eb, int max_m, int max_n, int kcap, bool refine, bool defer) {
+  return make_layout(eb, 0, max_m, max_n, kcap, refine, defer).total;
 }
 
 size_t tableau_row_bytes(int eb, int max_n, int kcap) { return size_t(tab_ld(max_n, kcap, eb)) * size_t(eb); }
 
-template <typename T, bool SE>
-static cudaError_t prep(size_t smem) {
-  return cudaFuncSetAttribute(tableau_kernel<T, SE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+static const void *tableau_fn(bool fp64, bool se, bool defer) {
+  return fp64 ? reinterpret_cast<const void *>(&tableau_kernel<double, false, false>)
+       : defer ? reinterpret_cast<const void *>(&tableau_kernel<float, false, true>)
+       : se ? reinterpret_cast<const void *>(&tableau_kernel<float, true, false>)
+            : reinterpret_cast<const void *>(&tableau_kernel<float, false, false>);
 }
 
-cudaError_t tableau_max_ctas_per_sm(int eb, int threads, size_t smem, int *ctas) {
-  if (eb == 8) {
-    const cudaError_t e = prep<double, false>(smem);
-    return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, tableau_kernel<double, false>, threads, smem);
-  }
-  const cudaError_t e = prep<float, false>(smem);
-  return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, tableau_kernel<float, false>, threads, smem);
+cudaError_t tableau_max_ctas_per_sm(int eb, int threads, size_t smem, bool defer, int *ctas) {
+  const void *fn = tableau_fn(eb == 8, false, defer);
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, fn, threads, smem);
 }
 
-cudaError_t launch_tableau(const TableauParams &p, bool fp64, int grid, int threads, size_t smem, cudaStream_t s) {
-  if (threads < 32 || threads > kMaxThreads || (threads & 31) || grid < 1) return cudaErrorInvalidValue;
-  const bool se = !fp64 && p.rule == LPB_PIVOT_STEEPEST;
-  const cudaError_t e = fp64 ? prep<double, false>(smem) : se ? prep<float, true>(smem) : prep<float, false>(smem);
+cudaError_t launch_tableau(const TableauParams &p, bool fp64, bool defer, int grid, int threads, size_t smem, cudaStream_t s) {
+  if (threads < 32 || threads > (defer ? kDefThreads : kMaxThreads) || (threads & 31) || grid < 1) return cudaErrorInvalidValue;
+  const void *fn = tableau_fn(fp64, p.rule == LPB_PIVOT_STEEPEST, defer);
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  if (fp64) tableau_kernel<double, false><<<grid, threads, smem, s>>>(p);
-  else if (se) tableau_kernel<float, true><<<grid, threads, smem, s>>>(p);
-  else tableau_kernel<float, false><<<grid, threads, smem, s>>>(p);
-  return cudaGetLastError();
+  void *args[] = {const_cast<TableauParams *>(&p)};
+  return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, s);
 }
 
 }  // namespace lpb

@@ -1,6 +1,6 @@
-"""The kernel that keeps the pivots instead of a tableau (the planner's choice under the
-largest-coefficient rule) against the kernels that update a tableau after every pivot, and
-against the oracle.
+"""The kernel that keeps the pivots instead of a tableau, and the tableau kernel's deferred
+updates in Phase I (the planner's choices under the largest-coefficient rule), against the
+kernels that update a tableau after every pivot, and against the oracle.
 
 Both form every tableau value by the same operations in the same order, so statuses, pivot
 counts and bases are equal, bit for bit; the FP64 results, which are read straight off, are
@@ -83,6 +83,30 @@ def test_more_pivots_than_the_history_holds(solver, m, n, prec, rtol):
     assert np.all(np.abs(got["obj"] - ref["obj"])[ok] <= rtol * (1 + np.abs(ref["obj"][ok])))
     if prec == "fp64":
         assert np.array_equal(got["iters"], ref["iters"])
+    assert solver.sync_error() == 0
+
+
+# Both sides of the deferred updates' least size, of 128 and 256 rows or columns (the CTA's
+# threads), and of a row's last vector; pivots from fewer than wait at once to many sweeps.
+@pytest.mark.parametrize("m,n", [(30, 38), (33, 41), (60, 20), (64, 64), (90, 97), (128, 60), (60, 131), (200, 200),
+                                 (258, 30), (30, 259)])
+@pytest.mark.parametrize("prec", ["fp32", "fp32_refine"])
+def test_deferred_updates_in_phase_one(solver, m, n, prec):
+    """Two-phase LPs (infeasible and unbounded ones among them): the same pivots, statuses
+    and bases as with a full update after every pivot."""
+    sb = synth.type2(80, m, n, seed=m + n, frac_infeasible=0.1, frac_unbounded=0.1)
+    batch = to_device(sb)
+    got = host(solver.solve(batch, prec=prec))
+    ref = host(solver.solve(batch, prec=prec, kernel=GMEM))
+    for name in ("status", "iters", "basis"):
+        assert np.array_equal(got[name], ref[name]), name
+    for name in ("obj", "x", "y"):
+        if prec == "fp32":
+            assert np.array_equal(got[name], ref[name], equal_nan=True), name
+        else:
+            fin = np.isfinite(ref[name])
+            assert np.array_equal(got[name][~fin], ref[name][~fin])
+            np.testing.assert_allclose(got[name][fin], ref[name][fin], rtol=1e-9, atol=1e-9)
     assert solver.sync_error() == 0
 
 
