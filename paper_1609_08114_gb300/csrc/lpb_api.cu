@@ -287,14 +287,15 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // tableau kernel, so it lies above what LPs with a bound on every variable take
 // (200 x 100, 64 pivots on average, 100 at most: 10,000 in 9.5 ms with none
 // handed on, 16 ms with 45% handed on, 17.5 ms all by the tableau kernel).
-void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, Pass *p) {
-  if (o->kernel != LPB_KERNEL_AUTO || o->threads != 0 || o->reg_warps != 0) return;
+void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int shared, Pass *p) {
+  if ((o->kernel != LPB_KERNEL_AUTO && shared != 2) || o->threads != 0 || o->reg_warps != 0) return;
   if (o->pivot_rule != LPB_PIVOT_LPC || p->pack > 0) return;
   const int kind = p->fp64 ? LAZY_FP64 : (p->warp || p->reg >= 0) ? LAZY_SMALL : LAZY_LARGE;
   const int eb = p->fp64 ? 8 : 4;
   LazyShape q{};
   q.max_m = p->lim_m;
   q.max_n = p->lim_n;
+  q.shared = shared != 0;
   const int mn = q.max_m < q.max_n ? q.max_m : q.max_n;
   q.kmax = (64 + mn / 2 + 3) & ~3;
   q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : kind == LAZY_SMALL ? 6 + mn / 10 : 8 + mn / 4;
@@ -321,7 +322,7 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, Pa
 // `plain`: full updates after every pivot in every pass (no history slots, more
 // rows in shared memory).
 lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, bool basis_given,
-                  Plan *pl, bool plain = false) {
+                  Plan *pl, bool plain = false, int shared = 0) {
   if (!b || !o) return LPB_EINVAL;
   if (b->count < 0) return LPB_EINVAL;
   if (b->max_m < 1 || b->max_n < 1 || b->max_m > kMaxDim || b->max_n > kMaxDim) return LPB_EUNSUPPORTED;
@@ -453,7 +454,7 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
     np = 1;
   }
   if (!plain)
-    for (int i = 0; i < np; ++i) lazy_pass(d, b, o, &pl->pass[i]);
+    for (int i = 0; i < np; ++i) lazy_pass(d, b, o, shared, &pl->pass[i]);
   {                                // LPs that need more artificial columns (Phase I)
     Pass &p = pl->pass[np];
     if ((e = make_pass(d, b, &og, !fp32, b->max_m, mode, plain, &p)) != LPB_OK) return e;
@@ -525,9 +526,9 @@ DeviceInfo device_info(const lpb_handle *h) { return DeviceInfo{h->sms, h->smem_
 namespace lpb {
 
 lpb_err solve_workspace_bytes(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
-                              bool basis_given, size_t *bytes, bool least) {
+                              bool basis_given, size_t *bytes, bool least, int shared) {
   Plan pl;
-  const lpb_err e = make_plan(d, b, o, basis_given, &pl, least);
+  const lpb_err e = make_plan(d, b, o, basis_given, &pl, least, shared);
   if (e != LPB_OK) return e;
   *bytes = pl.total;
   return LPB_OK;
@@ -539,7 +540,7 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
                   int shared) {
   if (kernels) *kernels = 0;
   Plan pl;
-  lpb_err e = make_plan(d, b, o, r->basis != nullptr, &pl);
+  lpb_err e = make_plan(d, b, o, r->basis != nullptr, &pl, false, shared);
   if (e != LPB_OK) return e;
   if (ws_bytes < pl.total) {       // less scratch than asked for: full updates, which need less
     pl = Plan();
@@ -656,7 +657,8 @@ void chunk_range(const int64_t *off, int k0, int k1, F len, int64_t *lo, int64_t
   *hi = off[k1 - 1] + len(k1 - 1);
 }
 
-lpb_err make_host_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int chunk, HostPlan *hp) {
+lpb_err make_host_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int chunk, HostPlan *hp,
+                       bool least = false) {
   if (!b || !o || chunk < 1) return LPB_EINVAL;
   if (b->count < 0) return LPB_EINVAL;
   if (b->count > 0 && (!b->m || !b->n || !b->a_off || !b->b_off || !b->c_off || !b->A || !b->b || !b->c))
@@ -684,7 +686,7 @@ lpb_err make_host_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_option
   }
   lpb_batch cb = *b;
   cb.count = hp->chunk;
-  const lpb_err e = solve_workspace_bytes(d, &cb, o, false, &hp->solve_ws);
+  const lpb_err e = solve_workspace_bytes(d, &cb, o, false, &hp->solve_ws, least);
   if (e != LPB_OK) return e;
   const size_t es = b->dtype == LPB_DTYPE_F64 ? 8 : 4;
   const size_t ch = size_t(hp->chunk);
@@ -730,9 +732,13 @@ __global__ void fill_shared_meta(int32_t *m, int32_t *n, int64_t *a_off, int64_t
 }
 
 // Options of a shared-constraint solve: FP32 solves that fit a register
-// template run on the register kernel over the identity work list, so that
-// each CTA takes consecutive objectives and can start each from the basis of
-// the one before.
+// template run with the register kernel's arithmetic over the identity work
+// list, so that each CTA takes consecutive objectives and can start each from
+// the basis of the one before: on the register kernel, or (lazy_pass) on the
+// kernel that keeps the pivots, whose warm start runs the new objective through
+// them (50,000 objectives at 100 x 100, ms on the register kernel and on this
+// one: independent directions 4.62 and 1.92, a sweep 1.64 and 0.76; 30,000 at
+// 40 x 30: 1.27 and 0.30, 0.78 and 0.20).
 lpb_options shared_options(const lpb_options *o, int m, int n) {
   lpb_options os = *o;
   if (o->prec != LPB_FP64 && o->kernel == LPB_KERNEL_AUTO && o->threads == 0 &&
@@ -745,8 +751,14 @@ struct SharedPlan {
   size_t o_m = 0, o_n = 0, o_ao = 0, o_bo = 0, o_co = 0, o_yo = 0, o_ws = 0, solve_ws = 0, total = 0;
 };
 
-lpb_err make_shared_plan(const DeviceInfo &d, int m, int n, int dtype, int64_t count, const lpb_options *o,
-                         SharedPlan *sp) {
+// Whether the planner is free to give a shared-constraint solve the kernel that
+// keeps the pivots (its warm starts are that kernel's own).
+int shared_mode(const lpb_options *o) {
+  return o->kernel == LPB_KERNEL_AUTO && o->threads == 0 && o->reg_warps == 0 ? 2 : 1;
+}
+
+lpb_err make_shared_plan(const DeviceInfo &d, int m, int n, int dtype, int64_t count, const lpb_options *o, int shared,
+                         bool least, SharedPlan *sp) {
   if (!o || m < 1 || n < 1 || count < 0 || count > INT32_MAX) return LPB_EINVAL;
   lpb_batch pb{};
   pb.count = int32_t(count);
@@ -755,7 +767,7 @@ lpb_err make_shared_plan(const DeviceInfo &d, int m, int n, int dtype, int64_t c
   pb.min_m = m;            // every LP of the batch has the one size m x n
   pb.min_n = n;
   pb.dtype = dtype;
-  const lpb_err e = solve_workspace_bytes(d, &pb, o, false, &sp->solve_ws);
+  const lpb_err e = solve_workspace_bytes(d, &pb, o, false, &sp->solve_ws, least, shared);
   if (e != LPB_OK) return e;
   const size_t c = size_t(count > 0 ? count : 1);
   size_t off = 0;
@@ -844,7 +856,8 @@ struct BoundedPlan {
   size_t o_A = 0, o_b = 0, o_y = 0, o_m = 0, o_n = 0, o_ao = 0, o_bo = 0, o_co = 0, o_ws = 0, solve_ws = 0, total = 0;
 };
 
-lpb_err make_bounded_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, BoundedPlan *bp) {
+lpb_err make_bounded_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, BoundedPlan *bp,
+                          bool least = false) {
   if (!b || !o || b->count < 0 || b->max_m < 1 || b->max_n < 1) return LPB_EINVAL;
   if (b->dtype != LPB_DTYPE_F64) return LPB_EUNSUPPORTED;   // the reduced LP reads the caller's c as FP64
   if (b->max_m + b->max_n > kMaxDim) return LPB_EUNSUPPORTED;
@@ -852,7 +865,7 @@ lpb_err make_bounded_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_opt
   rb.min_m = rb.min_n = 0;      // the reduced LPs have m + n rows
   rb.max_m = b->max_m + b->max_n;
   rb.dtype = LPB_DTYPE_F64;
-  const lpb_err e = solve_workspace_bytes(d, &rb, o, false, &bp->solve_ws);
+  const lpb_err e = solve_workspace_bytes(d, &rb, o, false, &bp->solve_ws, least);
   if (e != LPB_OK) return e;
   const size_t c = size_t(b->count > 0 ? b->count : 1), rows = size_t(b->max_m + b->max_n);
   size_t off = 0;
@@ -1026,6 +1039,10 @@ lpb_err lpb_solve_host(lpb_handle *h, const lpb_batch *b, const lpb_options *o, 
   HostPlan hp;
   lpb_err e = make_host_plan(d, b, o, chunk, &hp);
   if (e != LPB_OK) return e;
+  if (ws_bytes < hp.total) {       // less than asked for: full updates (see run_solve)
+    hp = HostPlan();
+    if ((e = make_host_plan(d, b, o, chunk, &hp, true)) != LPB_OK) return e;
+  }
   if (ws_bytes < hp.total || !ws) return LPB_ENOMEM;
   if (reinterpret_cast<uintptr_t>(ws) & 255) return LPB_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -1116,7 +1133,7 @@ lpb_err lpb_workspace_size_shared(lpb_handle *h, int32_t m, int32_t n, int32_t d
   if (!ds.ok()) return LPB_ECUDA;
   SharedPlan sp;
   const lpb_options os = shared_options(o, m, n);
-  const lpb_err e = make_shared_plan(device_info(h), m, n, dtype, count, &os, &sp);
+  const lpb_err e = make_shared_plan(device_info(h), m, n, dtype, count, &os, shared_mode(o), false, &sp);
   if (e != LPB_OK) return e;
   *bytes = sp.total;
   return LPB_OK;
@@ -1134,8 +1151,13 @@ lpb_err lpb_solve_shared(lpb_handle *h, int32_t m, int32_t n, int32_t dtype, con
   const DeviceInfo d = device_info(h);
   SharedPlan sp;
   const lpb_options os = shared_options(o, m, n);
+  const int shared = shared_mode(o);
   o = &os;
-  lpb_err e = make_shared_plan(d, m, n, dtype, count, o, &sp);
+  lpb_err e = make_shared_plan(d, m, n, dtype, count, o, shared, false, &sp);
+  if (e == LPB_OK && ws_bytes < sp.total) {     // less than asked for: full updates (see run_solve)
+    sp = SharedPlan();
+    e = make_shared_plan(d, m, n, dtype, count, o, shared, true, &sp);
+  }
   if (e != LPB_OK) return e;
   if (ws_bytes < sp.total || !ws) return LPB_ENOMEM;
   if (reinterpret_cast<uintptr_t>(ws) & 255) return LPB_EINVAL;
@@ -1164,7 +1186,7 @@ lpb_err lpb_solve_shared(lpb_handle *h, int32_t m, int32_t n, int32_t dtype, con
   bt.b = b;
   bt.c = C;
   return run_solve(d, h->d_ctr, h->d_err, &bt, o, r, w + sp.o_ws, sp.solve_ws, s, nullptr, nullptr,
-                   &h->last_kernels, 0, dyo, 1);
+                   &h->last_kernels, 0, dyo, shared);
 }
 
 lpb_err lpb_workspace_size_bounded(lpb_handle *h, const lpb_batch *b, const lpb_options *o, size_t *bytes) {
@@ -1193,6 +1215,10 @@ lpb_err lpb_solve_bounded(lpb_handle *h, const lpb_batch *b, const void *l, cons
   BoundedPlan bp;
   lpb_err e = make_bounded_plan(d, b, o, &bp);
   if (e != LPB_OK) return e;
+  if (ws_bytes < bp.total) {       // less than asked for: full updates (see run_solve)
+    bp = BoundedPlan();
+    if ((e = make_bounded_plan(d, b, o, &bp, true)) != LPB_OK) return e;
+  }
   if (ws_bytes < bp.total || !ws) return LPB_ENOMEM;
   if (reinterpret_cast<uintptr_t>(ws) & 255) return LPB_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -442,6 +442,7 @@ int warp_tab_bytes(int max_m, int max_n);
 struct LazyShape {
   int max_m, max_n;
   int ks, kmax;                // history entries in shared memory; pivots at most
+  bool shared;                 // objectives of one polytope
 };
 struct LazyLayout {
   int hs;                      // elements of a history entry
@@ -477,7 +478,7 @@ constexpr int kCounters = 8;   // device int32 work queues and list lengths of o
 // `least`: of the plan with full updates, which run_solve takes when the
 // workspace holds no more.
 lpb_err solve_workspace_bytes(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
-                              bool basis_given, size_t *bytes, bool least = false);
+                              bool basis_given, size_t *bytes, bool least = false, int shared = 0);
 // Zero `ctr` (kCounters device ints) and launch every pass of a solve on `s`,
 // with scratch from `ws`.  prof_ev (3 pairs) / prof_ran (3 flags) may be null.
 // lp_base: batch index of the batch's LP 0 (a chunk of a larger batch), which

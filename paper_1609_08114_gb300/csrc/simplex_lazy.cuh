@@ -29,6 +29,10 @@
 //     correction B^-1 r by running the pivots on r as another right-hand side,
 //     its transpose as another objective row (k (m + n) operations); the KKT
 //     certificate of the other kernels.
+//   * Objectives of one polytope (lpb_solve_shared): a CTA takes consecutive ones
+//     and starts each from the basis of the one before, whose history, right-hand
+//     side and variables it keeps: the new objective row is -c run through the
+//     pivots (k n operations).
 #pragma once
 #include <type_traits>
 
@@ -37,6 +41,11 @@
 namespace lpb {
 
 namespace {
+
+// Objectives of one polytope: consecutive ones claimed at a time, and warm starts
+// between two cold ones.
+constexpr int kShareChunk = 16;
+constexpr int kWarmMax = 32;
 
 __device__ __forceinline__ float neg(float v) { return -v; }
 __device__ __forceinline__ double neg(double v) { return neg_bits(v); }
@@ -77,6 +86,14 @@ template <typename T> using Img = std::conditional_t<sizeof(T) == 8, unsigned lo
 // conversion runs on the slow FP64 unit).
 __device__ __forceinline__ double widen(double v) { return v; }
 __device__ __forceinline__ double widen(float v) { return f2d_exact(v); }
+// The same for a finite entry of A in the FP64 products, without branches:
+// magnitudes below the smallest normal float count as zero.
+__device__ __forceinline__ double widen_a(double v) { return v; }
+__device__ __forceinline__ double widen_a(float v) {
+  const unsigned u = __float_as_uint(v), mag = u & 0x7fffffffu;
+  const bool z = mag < 0x00800000u;
+  return __hiloint2double(int((u & 0x80000000u) | (z ? 0u : (mag >> 3) + (896u << 20))), int(z ? 0u : u << 29));
+}
 
 // Entry `i` of the LP's A as the tableau's type: RN = false truncates FP64 to
 // FP32 (as the register kernel does), RN = true rounds (as the tableau kernel does).
@@ -96,11 +113,9 @@ __device__ __forceinline__ T a_in(const void *A, int i) {
 }
 
 // Largest magnitude image (FP64: the high word, FP32: the word) of the LP's
-// `cnt` entries of A, by 16-byte loads, kU in flight per thread.  `stop`, asked
-// once while the first are on their way, may end it (an LP that goes elsewhere
-// anyway is not read through).
-template <bool F64, int NT, typename F>
-__device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid, F &&stop) {
+// `cnt` entries of A, by 16-byte loads, kU in flight per thread.
+template <bool F64, int NT>
+__device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid) {
   constexpr int ES = F64 ? 8 : 4, PER = 16 / ES, kU = 8;
   const unsigned char *p = static_cast<const unsigned char *>(A);
   int head = int((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / ES;
@@ -116,25 +131,10 @@ __device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid, F &&
     if (!F64) amax = max(amax, max(v.x & 0x7fffffffu, v.z & 0x7fffffffu));
     amax = max(amax, max(v.y & 0x7fffffffu, v.w & 0x7fffffffu));
   };
-  uint4 v[kU];
-  if (nv > 0) {                    // the first loads; past the end the last vector again
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v[u] = __ldg(v4 + min(tid + u * NT, nv - 1));
-  }
-  if (stop()) return 0u;
-  if (nv > 0) {
-#pragma unroll
-    for (int u = 0; u < kU; ++u) fold(v[u]);
-  }
-  int k = tid + kU * NT;
+  int k = tid;
 #pragma unroll 1
-  for (; k + (kU - 1) * NT < nv; k += kU * NT) {
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v[u] = __ldg(v4 + k + u * NT);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) fold(v[u]);
-  }
-  if (k - tid < nv) {
+  for (; k - tid < nv; k += kU * NT) {         // past the end the last vector again
+    uint4 v[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) v[u] = __ldg(v4 + min(k + u * NT, nv - 1));
 #pragma unroll
@@ -187,7 +187,9 @@ __host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warp
 // T: the tableau's type; W warps and R rows (columns) per thread; F64: the
 // input's type; RN: the tableau kernel's arithmetic (input rounded, exact
 // ratios) instead of the register kernel's (input truncated, approximate ones).
-template <typename T, int W, int R, int MINB, bool F64, bool RN>
+// SHARED: objectives of one polytope, with warm starts (its own instantiation,
+// so that the others carry none of it).
+template <typename T, int W, int R, int MINB, bool F64, bool RN, bool SHARED>
 __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams P, const LazyLayout L) {
   extern __shared__ __align__(16) unsigned char lz_smem[];
   using In = std::conditional_t<F64, double, float>;
@@ -243,9 +245,15 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     c_ = __ldg(P.B.c_off + lp_);
   };
   // Claims are made one LP ahead; a CTA of several warps passes them on in
-  // shared memory, before the barrier of the vote on the input.
+  // shared memory, before the barrier of the vote on the input.  Objectives of
+  // one polytope (P.shared) are claimed kShareChunk consecutive ones at a time.
+  auto claim = [&](int cur) -> int {
+    if (!SHARED) return atomicAdd(P.queue, 1);
+    if (cur >= 0 && (cur + 1) % kShareChunk != 0 && cur + 1 < nitems) return cur + 1;
+    return atomicAdd(P.queue, 1) * kShareChunk;
+  };
   int item = 0;
-  if (tid == 0) item = atomicAdd(P.queue, 1);
+  if (tid == 0) item = claim(-1);
   if constexpr (W == 1) {
     item = __shfl_sync(kFull, item, 0);
   } else {
@@ -257,19 +265,32 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   int lp = 0, m = 0, n = 0;
   long long aoff = 0, boff = 0, coff = 0;
   if (item < nitems) read_desc(item, lp, m, n, aoff, boff, coff);
+  // What a warm start of the next objective of one polytope keeps (SHARED).
+  T rhs[R], obj[R];
+  unsigned bkey[R], nkey[R];       // keys of each row and column: its variable << kIdxBits | its index
+  int rst[R], cst[R];              // last pivot on each row and column, -1: none
+  unsigned long long bm = 0ull;    // largest |b| (its bits)
+  int held = 0;                    // pivots in the history
+  int warm_run = 0;                // objectives since a cold start; -1: the history is no basis of this polytope
+  bool scanned = false;            // the shared A is known to be finite
+  int cold_left = 0;               // objectives to start cold, since a warm start took many pivots
 #pragma unroll 1
   while (item < nitems) {
     int nitem = 0;
-    if (tid == 0) nitem = atomicAdd(P.queue, 1);
+    if (tid == 0) nitem = claim(item);
     // ---- admission: sizes, b >= 0, finite data in the tableau's range ----
     const In *A = static_cast<const In *>(P.B.A) + aoff;
     const In *bg = static_cast<const In *>(P.B.b) + boff, *cg = static_cast<const In *>(P.B.c) + coff;
     const bool fits = fits_lp(m, n);
     int bad = !fits;
-    unsigned long long bm = 0ull, cm = 0ull;
-    T rhs[R], obj[R];
-    unsigned bkey[R], nkey[R];     // keys of each row and column: its variable << kIdxBits | its index
-    int rst[R], cst[R];            // last pivot on each row and column, -1: none
+    // A warm start keeps the basis of the objective before: while few pivots
+    // lead to it (chains run over all of them), for a bounded number of
+    // objectives (FP32 round-off grows with the pivots), and not where the
+    // directions have little to do with one another.
+    const bool warm = SHARED && P.mode == MODE_FP32_REFINE && warm_run >= 0 && warm_run < kWarmMax && held > 0 &&
+                      held <= ks && cold_left == 0;
+    if (SHARED && cold_left > 0) --cold_left;
+    unsigned long long cm = 0ull;
     int ic[R], jc[R];              // own rows and columns; past the end the last one (read, never used)
     bool in_m[R], in_n[R];
     if (fits) {                    // (the same in every thread)
@@ -280,36 +301,43 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         in_n[r] = i < n;
         ic[r] = min(i, m - 1);
         jc[r] = min(i, n - 1);
-        bkey[r] = unsigned(((n + i) << kIdxBits) | i);
-        nkey[r] = unsigned((i << kIdxBits) | i);
-        rst[r] = -1;
-        cst[r] = -1;
         const In b = __ldg(bg + ic[r]), c = __ldg(cg + jc[r]);
         const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(widen(b)));
         const unsigned long long a = u & 0x7fffffffffffffffull;
         const unsigned long long v = static_cast<unsigned long long>(__double_as_longlong(widen(c))) & 0x7fffffffffffffffull;
         bad |= int((u >> 63) != 0ull && a != 0ull);
+        if (r == 0) bm = 0ull;
         bm = a > bm ? a : bm;
         cm = v > cm ? v : cm;
+        T bt;
         if constexpr (kD) {
-          rhs[r] = widen(b);
+          bt = widen(b);
           obj[r] = neg(widen(c));
         } else if constexpr (!F64) {
-          rhs[r] = b;
+          bt = b;
           obj[r] = -c;
         } else if constexpr (RN) {
-          rhs[r] = __double2float_rn(b);
+          bt = __double2float_rn(b);
           obj[r] = -__double2float_rn(c);
-          bad |= int(!isfinite(rhs[r])) | int(!isfinite(obj[r]));
+          bad |= int(!isfinite(bt)) | int(!isfinite(obj[r]));
         } else {
-          rhs[r] = d2f_tile(b, bad);
+          bt = d2f_tile(b, bad);
           obj[r] = -d2f_tile(c, bad);
+        }
+        if (!warm) {
+          rhs[r] = bt;
+          bkey[r] = unsigned(((n + i) << kIdxBits) | i);
+          nkey[r] = unsigned((i << kIdxBits) | i);
+          rst[r] = -1;
+          cst[r] = -1;
         }
       }
       bad |= int(bm >= kInf) | int(cm >= kInf);
-      const unsigned amax = scan_a<F64, NT>(A, m * n, tid, [&]() { return any(bad); });
-      // Not finite, or (FP32) so large that rounding could leave the float range.
-      bad |= int(amax >= (F64 ? (kD ? 0x7ff00000u : 0x47efffffu) : 0x7f800000u));
+      if ((!SHARED || !scanned) && !any(bad)) {      // (an LP for Phase I is not read through)
+        const unsigned amax = scan_a<F64, NT>(A, m * n, tid);
+        // Not finite, or (FP32) so large that rounding could leave the float range.
+        bad |= int(amax >= (F64 ? (kD ? 0x7ff00000u : 0x47efffffu) : 0x7f800000u));
+      }
     }
     bm = warp_max_u64(bm);
     cm = warp_max_u64(cm);
@@ -334,10 +362,16 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       }
     };
     if (bad) {
+      warm_run = -1;
       defer();
       next();
       continue;
     }
+    if constexpr (SHARED) {
+      scanned = true;
+      warm_run = warm ? warm_run + 1 : 0;
+    }
+    if (!warm) held = 0;
 
     // The block's best candidate: least image o[], then least key (kNone: no
     // candidate), with the values va, vb and the last pivot of its owner.  One
@@ -382,10 +416,58 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     // Entry s of the history.
     auto entry = [&](int s) -> const T * { return s < ks ? hist + s * hs : spill + (s - ks) * hs; };
 
+    // The history's pivots on an objective row w (by column), and on a right-hand
+    // side v (by row) where there is one.
+    auto through_pivots = [&](float *v, float *w) __attribute__((always_inline)) {
+      float *bc = reinterpret_cast<float *>(sums);       // [2 parities][v_l, w_e] (several warps)
+      auto publish = [&](int s) {
+        const int l = int(ats[s] >> 16), e = int(ats[s] & 0xffffu);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (v && tid + NT * r == l) bc[2 * (s & 1)] = v[r];
+          if (tid + NT * r == e) bc[2 * (s & 1) + 1] = w[r];
+        }
+      };
+      if (W > 1 && held > 0) publish(0);
+#pragma unroll 1
+      for (int s = 0; s < held; ++s) {
+        const T *h = entry(s);
+        const int l = int(ats[s] >> 16), e = int(ats[s] & 0xffffu);
+        float vl = 0.f, fm;
+        if constexpr (W == 1) {
+          float x = w[0], y = v ? v[0] : 0.f;
+#pragma unroll
+          for (int r = 1; r < R; ++r) {
+            const float xr = w[r], yr = v ? v[r] : 0.f;
+            x = (e >> 5) == r ? xr : x;
+            y = (l >> 5) == r ? yr : y;
+          }
+          if (v) vl = __shfl_sync(kFull, y, l & 31);
+          fm = __shfl_sync(kFull, x, e & 31) * float(rps[s]);
+        } else {
+          __syncthreads();
+          vl = bc[2 * (s & 1)];
+          fm = bc[2 * (s & 1) + 1] * float(rps[s]);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int i = tid + NT * r;
+          if (v) v[r] = fmaf(-float(h[ic[r]]), vl, i == l ? -0.f : v[r]);
+          w[r] = fmaf(-fm, float(h[pn + jc[r]]), i == e ? -0.f : w[r]);
+        }
+        if (W > 1 && s + 1 < held) publish(s + 1);
+      }
+      if constexpr (W > 1) __syncthreads();
+    };
+
     // ---- Steps 1-3 ----
     const int max_iter = P.max_iter > 0 ? P.max_iter : 50 * (m + n);
     int iters = 0, status = LPB_OPTIMAL, degenerate_run = 0;
     T z = T(0);
+    if (warm) {                    // the new objective row on the basis kept: -c through its pivots
+      sync();
+      if constexpr (SHARED) through_pivots(nullptr, obj);
+    }
     bool bland = false, over = false;
 #pragma unroll 1
     for (;;) {
@@ -398,7 +480,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       const int e = int(col.key) & kIdxMask, cse = col.last;
       // Column e: from A or from the pivot that last stood on it, then the pivots since.
       T a[R];
-      const int e1 = iters < ks ? iters : ks;
+      const int e1 = held < ks ? held : ks;
       {
         int s = cse + 1;
         if (cse < 0) {
@@ -417,7 +499,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
           for (int r = 0; r < R; ++r) a[r] = mul_add(neg(h[ic[r]]), pe, s == rst[r] ? neg_zero<T>() : a[r]);
         }
 #pragma unroll 1
-        for (; s < iters; ++s) {
+        for (; s < held; ++s) {
           const T *h = spill + (s - ks) * hs;
           const T pe = h[pn + e];
 #pragma unroll
@@ -476,7 +558,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       const Cand<T> row = choose(1, o, bkey, a, rhs, rst);
       if (row.o == kNone) { status = LPB_UNBOUNDED; break; }
       if (iters >= max_iter) { status = LPB_ITER_LIMIT; break; }
-      if (iters >= L.kmax) { over = true; break; }
+      if (held >= L.kmax) { over = true; break; }
       const int l = int(row.key) & kIdxMask, rsl = row.last;
       const T rp = recip(row.a), bl = row.b;
       // Row l: from A or from the pivot that last stood on it, then the pivots since.
@@ -500,7 +582,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
           for (int r = 0; r < R; ++r) p[r] = mul_add(nf, h[pn + jc[r]], s == cst[r] ? neg_zero<T>() : p[r]);
         }
 #pragma unroll 1
-        for (; s < iters; ++s) {
+        for (; s < held; ++s) {
           const T *h = spill + (s - ks) * hs;
           const T nf = neg(h[l]);
 #pragma unroll
@@ -509,7 +591,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       }
       // Step 3 on the right-hand side and the objective row, and the pivot into
       // the history.
-      T *h = iters < ks ? hist + iters * hs : spill + (iters - ks) * hs;
+      T *h = held < ks ? hist + held * hs : spill + (held - ks) * hs;
       const T fm = col.a * rp;
       z = mul_add(neg(fm), bl, z);
 #pragma unroll
@@ -522,12 +604,13 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         obj[r] = mul_add(neg(fm), v, is_e ? neg_zero<T>() : obj[r]);
         if (in_m[r]) h[i] = f;
         if (in_n[r]) h[pn + i] = v;
-        if (is_l) { bkey[r] = (col.key & ~unsigned(kIdxMask)) | unsigned(l); rst[r] = iters; }
-        if (is_e) { nkey[r] = (row.key & ~unsigned(kIdxMask)) | unsigned(e); cst[r] = iters; }
+        if (is_l) { bkey[r] = (col.key & ~unsigned(kIdxMask)) | unsigned(l); rst[r] = held; }
+        if (is_e) { nkey[r] = (row.key & ~unsigned(kIdxMask)) | unsigned(e); cst[r] = held; }
       }
-      if (tid == 0) { rps[iters] = rp; ats[iters] = unsigned(l << 16 | e); }
+      if (tid == 0) { rps[held] = rp; ats[held] = unsigned(l << 16 | e); }
       if constexpr (W == 1) __syncwarp();     // (several warps: the next Step 1's barrier)
       ++iters;
+      ++held;
       if (!above(unimage(row.o), eps_p)) {
         if (++degenerate_run >= m + n) bland = true;
       } else {
@@ -542,7 +625,10 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       bvar[r] = int(bkey[r] >> kIdxBits);
       nvar[r] = int(nkey[r] >> kIdxBits);
     }
+    if (status == LPB_ITER_LIMIT) warm_run = -1;
+    if (warm && 2 * iters > held) cold_left = kShareChunk - 1;
     if (over) {
+      warm_run = -1;
       defer();
       next();
       continue;
@@ -671,8 +757,8 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
               const double x = xq[q + u], y = xq[kx + q + u];
 #pragma unroll
               for (int r = 0; r < R; ++r) {
-                sx[r] = fma(widen(va[u][r]), x, sx[r]);
-                sy[r] = fma(widen(vb[u][r]), y, sy[r]);
+                sx[r] = fma(widen_a(va[u][r]), x, sx[r]);
+                sy[r] = fma(widen_a(vb[u][r]), y, sy[r]);
               }
             }
         }
@@ -688,45 +774,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         }
         // Corrections with the FP32 basis inverse: the pivots on v as another
         // right-hand side, on w as another objective row.
-        if constexpr (W == 1) {
-#pragma unroll 1
-          for (int s = 0; s < iters; ++s) {
-            const T *h = entry(s);
-            const int l = int(ats[s] >> 16), e = int(ats[s] & 0xffffu);
-            const float vl = pick(v, l), fm = pick(w, e) * float(rps[s]);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-              v[r] = fmaf(-float(h[ic[r]]), vl, lane + 32 * r == l ? -0.f : v[r]);
-              w[r] = fmaf(-fm, float(h[pn + jc[r]]), lane + 32 * r == e ? -0.f : w[r]);
-            }
-          }
-        } else {
-          float *bc = reinterpret_cast<float *>(sums);       // [2 parities][v_l, w_e]
-          auto publish = [&](int s) {
-            const int l = int(ats[s] >> 16), e = int(ats[s] & 0xffffu);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-              if (tid + NT * r == l) bc[2 * (s & 1)] = v[r];
-              if (tid + NT * r == e) bc[2 * (s & 1) + 1] = w[r];
-            }
-          };
-          if (iters > 0) publish(0);
-#pragma unroll 1
-          for (int s = 0; s < iters; ++s) {
-            __syncthreads();
-            const T *h = entry(s);
-            const int l = int(ats[s] >> 16), e = int(ats[s] & 0xffffu);
-            const float vl = bc[2 * (s & 1)], fm = bc[2 * (s & 1) + 1] * float(rps[s]);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-              const int i = tid + NT * r;
-              v[r] = fmaf(-float(h[ic[r]]), vl, i == l ? -0.f : v[r]);
-              w[r] = fmaf(-fm, float(h[pn + jc[r]]), i == e ? -0.f : w[r]);
-            }
-            if (s + 1 < iters) publish(s + 1);
-          }
-          __syncthreads();
-        }
+        through_pivots(v, w);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           if (qi[r] >= 0) dv[qi[r]] = v[r];
@@ -832,6 +880,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         }
       }
     }
+    if (fail && opt) warm_run = -1;          // the next objective starts cold
     if (tid == 0) {
       P.R.status[lp] = fail ? STATUS_PENDING : LPB_OPTIMAL;
       if (!fail) P.R.obj[lp] = cx;
@@ -846,12 +895,20 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
 struct LazyConfig {
   int W, R;
   const void *f64, *f32;          // instantiations by input type
+  const void *s64, *s32;          // ... for objectives of one polytope, or null
 };
 
 template <typename T, int W, int R, int MINB, bool RN>
 constexpr LazyConfig lazy_config() {
-  return LazyConfig{W, R, reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN>),
-                    reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN>)};
+  constexpr bool kS = sizeof(T) == 4 && !RN;
+  return LazyConfig{W, R, reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, false>),
+                    reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN, false>),
+                    reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, kS>),
+                    reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN, kS>)};
+}
+
+inline const void *lazy_fn(const LazyConfig &c, int dtype, bool shared) {
+  return dtype == LPB_DTYPE_F64 ? (shared ? c.s64 : c.f64) : (shared ? c.s32 : c.f32);
 }
 
 // Smallest configuration of a table that holds LPs up to max_dim, or null.
@@ -870,7 +927,7 @@ cudaError_t lazy_occ(const LazyConfig (&t)[N], const LazyShape &q, int dtype, in
   *lay = lazy_layout<T>(q.max_m, q.max_n, c->W, c->R, q.ks, q.kmax);
   *threads = 32 * c->W;
   if (lay->bytes > 230000) return cudaSuccess;
-  const void *fn = dtype == LPB_DTYPE_F64 ? c->f64 : c->f32;
+  const void *fn = lazy_fn(*c, dtype, q.shared);
   const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lay->bytes);
   return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, fn, *threads, size_t(lay->bytes));
 }
@@ -879,7 +936,7 @@ template <int N>
 cudaError_t lazy_launch(const LazyConfig (&t)[N], const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s) {
   const LazyConfig *c = lazy_pick(t, p.lim_m > p.lim_n ? p.lim_m : p.lim_n);
   if (!c) return cudaErrorInvalidValue;
-  const void *fn = p.B.dtype == LPB_DTYPE_F64 ? c->f64 : c->f32;
+  const void *fn = lazy_fn(*c, p.B.dtype, p.shared != 0);
   const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.bytes);
   if (e != cudaSuccess) return e;
   void *args[] = {const_cast<TableauParams *>(&p), const_cast<LazyLayout *>(&lay)};

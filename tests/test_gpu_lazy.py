@@ -149,3 +149,24 @@ def test_less_workspace_than_its_slots(solver):
     for name in ("status", "iters", "basis"):
         assert np.array_equal(got[name], want[name]), name
     assert call(256) == _lib.ENOMEM
+
+
+@pytest.mark.parametrize("m,n", [(12, 9), (31, 33), (64, 65), (65, 30), (100, 100), (127, 21)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("turn", [None, 1e-3])
+def test_objectives_of_one_polytope(solver, m, n, dtype, turn):
+    """Warm starts (directions that turn slowly) and cold ones (independent directions, a
+    last chunk that is not full) against FP64 solves of the same objectives."""
+    r = np.random.default_rng(m + n)
+    A, b, _ = synth.type1(1, m, n, seed=m).lp(0)
+    count = 16 * 40 + 5
+    C = r.normal(size=(count, n)) if turn is None else (
+        r.uniform(0, 1, size=n)[None] + turn * np.arange(count)[:, None] * r.normal(size=n)[None])
+    args = [torch.tensor(v, device="cuda", dtype=dtype) for v in (A, b, C)]
+    got = host(solver.solve_shared(*args, prec="fp32_refine"))
+    ref = host(solver.solve_shared(*[a.double() for a in args], prec="fp64"))
+    assert np.array_equal(got["status"], ref["status"])
+    assert np.all(np.abs(got["obj"] - ref["obj"]) <= 1e-8 * (1 + np.abs(ref["obj"])))
+    if turn is not None:
+        assert got["iters"].mean() < 0.5 * ref["iters"].mean()
+    assert solver.sync_error() == 0
