@@ -4,7 +4,12 @@
 namespace lpb {
 
 namespace {
-const LazyConfig kTable[] = {lazy_config<float, 4, 2, 4, true>(), lazy_config<float, 8, 2, 2, true>(), lazy_config<float, 8, 4, 1, true>()};
+// Warps per LP, rows and columns per thread, CTAs per SM at least.
+const LazyConfig kTable[] = {
+    lazy_config<float, 4, 2, 4, true>(),
+    lazy_config<float, 8, 2, 2, true>(),
+    lazy_config<float, 8, 4, 1, true>(),
+};
 }  // namespace
 
 cudaError_t lazy_occupancy_large(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay) {

@@ -4,7 +4,12 @@
 namespace lpb {
 
 namespace {
-const LazyConfig kTable[] = {lazy_config<float, 1, 1, 16, false>(), lazy_config<float, 1, 2, 16, false>(), lazy_config<float, 2, 2, 8, false>()};
+// Warps per LP, rows and columns per thread, CTAs per SM at least.
+const LazyConfig kTable[] = {
+    lazy_config<float, 1, 1, 16, false>(),
+    lazy_config<float, 1, 2, 16, false>(),
+    lazy_config<float, 2, 2, 8, false>(),
+};
 }  // namespace
 
 cudaError_t lazy_occupancy_small(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay) {

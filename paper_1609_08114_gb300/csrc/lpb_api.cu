@@ -63,7 +63,14 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 enum ListKind { LIST_ALL = 0, LIST_CLASS = 1, LIST_DEFER = 2, LIST_RESOLVE = 3 };
 
-enum LazyKind { LAZY_NONE = 0, LAZY_SMALL = 1, LAZY_LARGE = 2, LAZY_FP64 = 3 };
+// The launches of the kernel that keeps the pivots.
+enum LazyKind { LAZY_SMALL = 0, LAZY_LARGE = 1, LAZY_FP64 = 2, LAZY_NONE = -1 };
+constexpr decltype(&lazy_occupancy_small) kLazyOccupancy[2][3] = {
+    {lazy_occupancy_small, lazy_occupancy_large, lazy_occupancy_fp64},
+    {lazy_occupancy_small_rpc, lazy_occupancy_large_rpc, lazy_occupancy_fp64_rpc}};
+constexpr decltype(&launch_lazy_small) kLaunchLazy[2][3] = {
+    {launch_lazy_small, launch_lazy_large, launch_lazy_fp64},
+    {launch_lazy_small_rpc, launch_lazy_large_rpc, launch_lazy_fp64_rpc}};
 
 struct Pass {
   bool fp64 = false, gmem = false;
@@ -277,7 +284,14 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 //   50,000 x 100                   4.19 -> 2.11    2,000 x 300    6.0 -> 1.8-2.1
 //   20,000 x 100, FP64 tableau    12.42 -> 1.38
 // The random rule takes over three times the pivots (45.6 against 13.3 at
-// 100 x 100), which favours a full update; it stays with the kernels that do one.
+// 100 x 100), so its chains are longer and a full update is the better one in
+// places: it comes here only with enough LPs to fill the GPU (300 x 100 FP64 0.98
+// and 1.31 ms, 600 x 120 FP32 input 0.30 and 0.75), in FP64 not for LPs of few
+// long rows (10,000 x 5 x 250 2.0 and 2.5), in FP32 up to 64 rows and columns or
+// above 127 rows with at most 128 columns (3,000 x 60 x 120 0.69 and 0.82, 600 x
+// 280 6.1 and 7.1), and not where the warp kernel had the pass (30,000 x 20 x 120
+// 1.6 and 2.1).  Where it does: 20,000 x 100 FP64 36.2 -> 9.3, 30,000 x 48 x 37
+// FP32 input 2.40 -> 0.60, 5,000 x 200 x 100 7.9 -> 3.3.
 // History entries in shared memory: about what a type-1 LP's pivots need (13 at
 // 100 x 100, 33 at 300 x 300); more of them cost LPs in flight (50,000 x 100:
 // 2.38 ms with 8, 2.18 with 12, 2.12 with 16, 2.18 with 20; 2,000 x 300: 2.37
@@ -289,23 +303,27 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // handed on, 16 ms with 45% handed on, 17.5 ms all by the tableau kernel).
 void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int shared, Pass *p) {
   if ((o->kernel != LPB_KERNEL_AUTO && shared != 2) || o->threads != 0 || o->reg_warps != 0) return;
-  if (o->pivot_rule != LPB_PIVOT_LPC || p->pack > 0) return;
+  if (o->pivot_rule == LPB_PIVOT_STEEPEST || p->pack > 0) return;
   const int kind = p->fp64 ? LAZY_FP64 : (p->warp || p->reg >= 0) ? LAZY_SMALL : LAZY_LARGE;
   const int eb = p->fp64 ? 8 : 4;
   LazyShape q{};
   q.max_m = p->lim_m;
   q.max_n = p->lim_n;
   q.shared = shared != 0;
+  const bool rpc = o->pivot_rule == LPB_PIVOT_RPC;
   const int mn = q.max_m < q.max_n ? q.max_m : q.max_n;
-  q.kmax = (64 + mn / 2 + 3) & ~3;
-  q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : kind == LAZY_SMALL ? 6 + mn / 10 : 8 + mn / 4;
+  if (rpc) {
+    const int mx = q.max_m > q.max_n ? q.max_m : q.max_n;
+    if (p->warp || b->count < 16 * d.sms) return;
+    if (kind == LAZY_FP64 ? mx > 8 * mn : kind == LAZY_SMALL ? mx > 64 : q.max_n > 128) return;
+  }
+  q.kmax = (64 + (rpc ? mn : mn / 2) + 3) & ~3;
+  q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL ? 6 + mn / 10 : 8 + mn / 4;
   const int most = 72 * 1024 / ((q.max_m + q.max_n) * eb);      // a third of an SM's shared memory
   if (q.ks > most) q.ks = most > 1 ? most : 1;
   int occ = 0, threads = 0;
   LazyLayout lay{};
-  const cudaError_t ce = kind == LAZY_FP64 ? lazy_occupancy_fp64(q, b->dtype, &occ, &threads, &lay)
-                       : kind == LAZY_SMALL ? lazy_occupancy_small(q, b->dtype, &occ, &threads, &lay)
-                                            : lazy_occupancy_large(q, b->dtype, &occ, &threads, &lay);
+  const cudaError_t ce = kLazyOccupancy[rpc][kind](q, b->dtype, &occ, &threads, &lay);
   if (ce != cudaSuccess) cudaGetLastError();
   if (ce != cudaSuccess || occ < 1) return;                      // too large: the pass stays as it is
   lay.tab = p->warp ? warp_tab_bytes(q.max_m, q.max_n) : 0;
@@ -607,9 +625,7 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
         p.eps_d = pl.eps_d64;
         break;
     }
-    const cudaError_t ce = ps.lazy == LAZY_SMALL ? launch_lazy_small(p, ps.lay, ps.grid, s)
-                         : ps.lazy == LAZY_LARGE ? launch_lazy_large(p, ps.lay, ps.grid, s)
-                         : ps.lazy == LAZY_FP64 ? launch_lazy_fp64(p, ps.lay, ps.grid, s)
+    const cudaError_t ce = ps.lazy != LAZY_NONE ? kLaunchLazy[o->pivot_rule == LPB_PIVOT_RPC][ps.lazy](p, ps.lay, ps.grid, s)
                          : ps.pack > 0 ? launch_pack(p, ps.pack, ps.grid, s)
                          : ps.warp ? launch_warp(p, ps.grid, ps.threads, ps.smem, s)
                          : ps.reg >= 0 ? launch_reg(p, ps.reg, ps.grid, ps.smem, s)

@@ -451,12 +451,17 @@ struct LazyLayout {
   int hist, rp, at, xq, dv, off, kr, flag, red;   // byte offsets
   int bytes;
 };
-cudaError_t lazy_occupancy_small(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay);
-cudaError_t lazy_occupancy_large(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay);
-cudaError_t lazy_occupancy_fp64(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay);
-cudaError_t launch_lazy_small(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
-cudaError_t launch_lazy_large(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
-cudaError_t launch_lazy_fp64(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
+// (_rpc: under the random entering rule.)
+#define LPB_LAZY(tag)                                                                                          \
+  cudaError_t lazy_occupancy_##tag(const LazyShape &q, int dtype, int *ctas, int *threads, LazyLayout *lay); \
+  cudaError_t launch_lazy_##tag(const TableauParams &p, const LazyLayout &lay, int grid, cudaStream_t s);
+LPB_LAZY(small)
+LPB_LAZY(small_rpc)
+LPB_LAZY(large)
+LPB_LAZY(large_rpc)
+LPB_LAZY(fp64)
+LPB_LAZY(fp64_rpc)
+#undef LPB_LAZY
 size_t hyperbox_smem_bytes(int n, int elem_bytes, bool shared_box);
 cudaError_t launch_hyperbox(const HyperboxParams &p, uint32_t *err, cudaStream_t s);
 // Backward kernel (backward.cu).

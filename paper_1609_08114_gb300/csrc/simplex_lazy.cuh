@@ -46,6 +46,7 @@ namespace {
 // between two cold ones.
 constexpr int kShareChunk = 16;
 constexpr int kWarmMax = 32;
+enum : int { kCommon = 0, kShared = 1, kRandom = 2 };
 
 __device__ __forceinline__ float neg(float v) { return -v; }
 __device__ __forceinline__ double neg(double v) { return neg_bits(v); }
@@ -187,15 +188,16 @@ __host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warp
 // T: the tableau's type; W warps and R rows (columns) per thread; F64: the
 // input's type; RN: the tableau kernel's arithmetic (input rounded, exact
 // ratios) instead of the register kernel's (input truncated, approximate ones).
-// SHARED: objectives of one polytope, with warm starts (its own instantiation,
-// so that the others carry none of it).
-template <typename T, int W, int R, int MINB, bool F64, bool RN, bool SHARED>
+// KIND: kShared (objectives of one polytope, with warm starts) and kRandom (the
+// random entering rule) are their own instantiations, so that the common one
+// carries none of either.
+template <typename T, int W, int R, int MINB, bool F64, bool RN, int KIND>
 __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams P, const LazyLayout L) {
   extern __shared__ __align__(16) unsigned char lz_smem[];
   using In = std::conditional_t<F64, double, float>;
   using Im = Img<T>;
   constexpr int NT = 32 * W, D = NT * R;
-  constexpr bool kD = sizeof(T) == 8;
+  constexpr bool kD = sizeof(T) == 8, SHARED = KIND == kShared;
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
   constexpr Im kNone = Im(~Im(0));
   T *hist = reinterpret_cast<T *>(lz_smem + L.hist);
@@ -474,7 +476,17 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       // Step 1: the most negative reduced cost (Bland: the lowest variable).
       Im o[R];
 #pragma unroll
-      for (int r = 0; r < R; ++r) o[r] = in_n[r] && above(neg(obj[r]), eps_d) ? (bland ? Im(0) : image(obj[r])) : kNone;
+      for (int r = 0; r < R; ++r) {
+        o[r] = in_n[r] && above(neg(obj[r]), eps_d) ? (bland ? Im(0) : image(obj[r])) : kNone;
+        // The random rule: the least key of the variable at this pivot (FP32: of
+        // its upper 31 bits, as the register kernel ranks; RN: of all but the one
+        // value that stands for no candidate).
+        if constexpr (KIND == kRandom)
+          if (o[r] != kNone && !bland) {
+            const unsigned key = rpc_key(P.seed, P.lp_base + lp, iters, int(nkey[r] >> kIdxBits));
+            o[r] = kD ? Im(key) : RN ? Im(min(key, 0xfffffffeu)) : Im(key >> 1);
+          }
+      }
       const Cand<T> col = choose(0, o, nkey, obj, obj, cst);
       if (col.o == kNone) break;
       const int e = int(col.key) & kIdxMask, cse = col.last;
@@ -895,14 +907,14 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
 struct LazyConfig {
   int W, R;
   const void *f64, *f32;          // instantiations by input type
-  const void *s64, *s32;          // ... for objectives of one polytope, or null
+  const void *s64, *s32;          // ... for objectives of one polytope (FP32, else the common ones)
 };
 
-template <typename T, int W, int R, int MINB, bool RN>
+template <typename T, int W, int R, int MINB, bool RN, int KIND = kCommon>
 constexpr LazyConfig lazy_config() {
-  constexpr bool kS = sizeof(T) == 4 && !RN;
-  return LazyConfig{W, R, reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, false>),
-                    reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN, false>),
+  constexpr int kS = sizeof(T) == 4 && !RN && KIND == kCommon ? int(kShared) : KIND;
+  return LazyConfig{W, R, reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, KIND>),
+                    reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN, KIND>),
                     reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, kS>),
                     reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN, kS>)};
 }

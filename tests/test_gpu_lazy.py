@@ -62,6 +62,21 @@ def test_same_pivots_as_the_full_update(solver, m, n, dtype, prec):
     assert solver.sync_error() == 0
 
 
+@pytest.mark.parametrize("m,n", [(40, 33), (64, 64), (130, 30)])
+@pytest.mark.parametrize("dtype,prec", [(torch.float32, "fp32"), (torch.float32, "fp32_refine"), (torch.float64, "fp64")])
+def test_same_pivots_under_the_random_rule(solver, m, n, dtype, prec):
+    """In a batch that fills the GPU (smaller ones keep the full update under this rule)."""
+    sb = synth.type1(2500, m, n, seed=m + 31 * n)
+    batch = _batch(sb, dtype)
+    full = GMEM if prec == "fp64" or max(m, n) > 127 else REG
+    got = host(solver.solve(batch, prec=prec, pivot_rule="rpc", seed=11))
+    ref = host(solver.solve(batch, prec=prec, pivot_rule="rpc", seed=11, kernel=full))
+    for name in ("status", "iters", "basis"):
+        assert np.array_equal(got[name], ref[name]), name
+    np.testing.assert_allclose(got["obj"], ref["obj"], rtol=1e-9)
+    assert solver.sync_error() == 0
+
+
 def _boxed(count, m, n, seed):
     """LPs of many pivots: rows of both signs and a bound on every variable."""
     r = np.random.default_rng(seed)
