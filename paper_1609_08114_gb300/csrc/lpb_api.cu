@@ -64,13 +64,14 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 enum ListKind { LIST_ALL = 0, LIST_CLASS = 1, LIST_DEFER = 2, LIST_RESOLVE = 3 };
 
 // The launches of the kernel that keeps the pivots.
-enum LazyKind { LAZY_SMALL = 0, LAZY_LARGE = 1, LAZY_FP64 = 2, LAZY_NONE = -1 };
-constexpr decltype(&lazy_occupancy_small) kLazyOccupancy[2][3] = {
-    {lazy_occupancy_small, lazy_occupancy_large, lazy_occupancy_fp64},
-    {lazy_occupancy_small_rpc, lazy_occupancy_large_rpc, lazy_occupancy_fp64_rpc}};
-constexpr decltype(&launch_lazy_small) kLaunchLazy[2][3] = {
-    {launch_lazy_small, launch_lazy_large, launch_lazy_fp64},
-    {launch_lazy_small_rpc, launch_lazy_large_rpc, launch_lazy_fp64_rpc}};
+// (LAZY_PACK: not under the random rule.)
+enum LazyKind { LAZY_SMALL = 0, LAZY_LARGE = 1, LAZY_FP64 = 2, LAZY_PACK = 3, LAZY_NONE = -1 };
+constexpr decltype(&lazy_occupancy_small) kLazyOccupancy[2][4] = {
+    {lazy_occupancy_small, lazy_occupancy_large, lazy_occupancy_fp64, lazy_occupancy_pack},
+    {lazy_occupancy_small_rpc, lazy_occupancy_large_rpc, lazy_occupancy_fp64_rpc, lazy_occupancy_pack}};
+constexpr decltype(&launch_lazy_small) kLaunchLazy[2][4] = {
+    {launch_lazy_small, launch_lazy_large, launch_lazy_fp64, launch_lazy_pack},
+    {launch_lazy_small_rpc, launch_lazy_large_rpc, launch_lazy_fp64_rpc, launch_lazy_pack}};
 
 struct Pass {
   bool fp64 = false, gmem = false;
@@ -283,6 +284,14 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 //   30,000 x 48 x 37, FP32 input   1.43 -> 0.28    50,000 x 64    1.46 -> 0.68
 //   50,000 x 100                   4.19 -> 2.11    2,000 x 300    6.0 -> 1.8-2.1
 //   20,000 x 100, FP64 tableau    12.42 -> 1.38
+// Of the several-LPs-per-warp kernel's passes those of plain FP32 with one or two
+// LPs per warp come here (100,000 LPs: 28 x 28 0.82 -> 0.25, 16 x 31 with FP32
+// input 0.87 -> 0.20, 15 x 15 0.22 -> 0.17, 12 x 12 0.19 -> 0.16, 8 x 8 0.15 ->
+// 0.13; 10,000 x 28 0.099 -> 0.052), from as many LPs on as take longer than the
+// host takes to plan and launch (10,000 x 12 0.048 and 0.050, 1,000 x 30 x 20
+// 0.047 and 0.049).  With four (m, n <= 7) that kernel's lanes are full.  Its refinement corrects by products with the final
+// tableau, which this kernel does not have: another rounding of the results, so
+// refined passes stay.
 // The random rule takes over three times the pivots (45.6 against 13.3 at
 // 100 x 100), so its chains are longer and a full update is the better one in
 // places: it comes here only with enough LPs to fill the GPU (300 x 100 FP64 0.98
@@ -303,8 +312,10 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // handed on, 16 ms with 45% handed on, 17.5 ms all by the tableau kernel).
 void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int shared, Pass *p) {
   if ((o->kernel != LPB_KERNEL_AUTO && shared != 2) || o->threads != 0 || o->reg_warps != 0) return;
-  if (o->pivot_rule == LPB_PIVOT_STEEPEST || p->pack > 0) return;
-  const int kind = p->fp64 ? LAZY_FP64 : (p->warp || p->reg >= 0) ? LAZY_SMALL : LAZY_LARGE;
+  if (o->pivot_rule == LPB_PIVOT_STEEPEST) return;
+  if (p->pack > 0 && (p->pack < 16 || p->mode != MODE_FP32 || o->pivot_rule != LPB_PIVOT_LPC || shared ||
+                      b->count < (p->pack == 32 ? 16 : 128) * d.sms)) return;
+  const int kind = p->pack > 0 ? LAZY_PACK : p->fp64 ? LAZY_FP64 : (p->warp || p->reg >= 0) ? LAZY_SMALL : LAZY_LARGE;
   const int eb = p->fp64 ? 8 : 4;
   LazyShape q{};
   q.max_m = p->lim_m;
@@ -318,7 +329,7 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
     if (kind == LAZY_FP64 ? mx > 8 * mn : kind == LAZY_SMALL ? mx > 64 : q.max_n > 128) return;
   }
   q.kmax = (64 + (rpc ? mn : mn / 2) + 3) & ~3;
-  q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL ? 6 + mn / 10 : 8 + mn / 4;
+  q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL || kind == LAZY_PACK ? 6 + mn / 10 : 8 + mn / 4;
   const int most = 72 * 1024 / ((q.max_m + q.max_n) * eb);      // a third of an SM's shared memory
   if (q.ks > most) q.ks = most > 1 ? most : 1;
   int occ = 0, threads = 0;

@@ -461,6 +461,7 @@ LPB_LAZY(large)
 LPB_LAZY(large_rpc)
 LPB_LAZY(fp64)
 LPB_LAZY(fp64_rpc)
+LPB_LAZY(pack)
 #undef LPB_LAZY
 size_t hyperbox_smem_bytes(int n, int elem_bytes, bool shared_box);
 cudaError_t launch_hyperbox(const HyperboxParams &p, uint32_t *err, cudaStream_t s);

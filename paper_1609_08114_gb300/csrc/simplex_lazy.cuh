@@ -33,6 +33,17 @@
 //     and starts each from the basis of the one before, whose history, right-hand
 //     side and variables it keeps: the new objective row is -c run through the
 //     pivots (k n operations).
+//
+// What bounds it, at 50,000 x 100 with FP64 input (4.19 ms on the kernel that updates
+// the whole tableau -> 2.06 ms, 0.30 of the copy bandwidth over the 83.6 KB that an LP
+// must move): the waits of each pivot on A's column and row, with 16 warps per SM to
+// hide them (scheduler slots 41% used, `long_scoreboard` 3.6 of 9 cycles per
+// instruction); 113 KB of DRAM traffic per LP, because L2 has let go of a part of A by
+// the time a pivot gathers from it.  That is also why an LP has two warps and eight LPs
+// an SM, and nothing is fetched ahead: one warp per LP and nine LPs, or fetching the next
+// LP, read A up to three times from DRAM (3.4 ms).  A one-time FP32 copy of A in shared
+// memory takes away the LPs in flight (2.45 ms at best).  FP64 tableau, 20,000 x 100
+// (12.4 -> 1.37 ms): the FP64 pipe, 69% busy.
 #pragma once
 #include <type_traits>
 
@@ -46,7 +57,7 @@ namespace {
 // between two cold ones.
 constexpr int kShareChunk = 16;
 constexpr int kWarmMax = 32;
-enum : int { kCommon = 0, kShared = 1, kRandom = 2 };
+enum : int { kCommon = 0, kShared = 1, kRandom = 2, kPacked = 3 };
 
 __device__ __forceinline__ float neg(float v) { return -v; }
 __device__ __forceinline__ double neg(double v) { return neg_bits(v); }
@@ -188,16 +199,17 @@ __host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warp
 // T: the tableau's type; W warps and R rows (columns) per thread; F64: the
 // input's type; RN: the tableau kernel's arithmetic (input rounded, exact
 // ratios) instead of the register kernel's (input truncated, approximate ones).
-// KIND: kShared (objectives of one polytope, with warm starts) and kRandom (the
-// random entering rule) are their own instantiations, so that the common one
-// carries none of either.
+// KIND: kShared (objectives of one polytope, with warm starts), kRandom (the
+// random entering rule) and kPacked (with RN: the arithmetic of the
+// several-LPs-per-warp kernel, ratios by the rounded reciprocal, and no
+// refinement) are their own instantiations, so that the common one carries none of them.
 template <typename T, int W, int R, int MINB, bool F64, bool RN, int KIND>
 __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams P, const LazyLayout L) {
   extern __shared__ __align__(16) unsigned char lz_smem[];
   using In = std::conditional_t<F64, double, float>;
   using Im = Img<T>;
   constexpr int NT = 32 * W, D = NT * R;
-  constexpr bool kD = sizeof(T) == 8, SHARED = KIND == kShared;
+  constexpr bool kD = sizeof(T) == 8, SHARED = KIND == kShared, PACKED = KIND == kPacked;
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
   constexpr Im kNone = Im(~Im(0));
   T *hist = reinterpret_cast<T *>(lz_smem + L.hist);
@@ -318,6 +330,9 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         } else if constexpr (!F64) {
           bt = b;
           obj[r] = -c;
+        } else if constexpr (PACKED) {
+          bt = d2f_rn(b);
+          obj[r] = -d2f_rn(c);
         } else if constexpr (RN) {
           bt = __double2float_rn(b);
           obj[r] = -__double2float_rn(c);
@@ -565,7 +580,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       } else {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          o[r] = in_m[r] && a[r] > eps_p ? image(T(RN ? rhs[r] / a[r] : rhs[r] * rcp_approx(float(a[r])))) : kNone;
+          o[r] = in_m[r] && a[r] > eps_p ? image(T(PACKED ? rhs[r] * recip(a[r]) : RN ? rhs[r] / a[r] : rhs[r] * rcp_approx(float(a[r])))) : kNone;
       }
       const Cand<T> row = choose(1, o, bkey, a, rhs, rst);
       if (row.o == kNone) { status = LPB_UNBOUNDED; break; }
@@ -652,7 +667,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         if (in_m[r]) bp[tid + NT * r] = bvar[r];
     }
     const bool opt = status == LPB_OPTIMAL;
-    if (kD || P.mode != MODE_FP32_REFINE) {          // results straight from the tableau; zeros where there is none
+    if (kD || PACKED || P.mode != MODE_FP32_REFINE) {          // results straight from the tableau; zeros where there is none
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int i = tid + NT * r, u = opt ? nvar[r] : i, v = opt ? bvar[r] : n + i;
@@ -673,7 +688,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       next();
       continue;
     }
-    if constexpr (!kD) {
+    if constexpr (!kD && !PACKED) {
     // ---- FP64 refinement and certificate ----
     // Numbers of the basic structurals (by row) and the non-basic slacks (by
     // column); there are as many of one as of the other.

@@ -18,7 +18,7 @@ from lp_helpers import compare, host, to_device
 
 pytestmark = pytest.mark.gpu
 
-GMEM, REG, WARP = 2, 3, 5
+GMEM, REG, PACK, WARP = 2, 3, 4, 5
 
 
 @pytest.fixture(scope="module")
@@ -60,6 +60,18 @@ def test_same_pivots_as_the_full_update(solver, m, n, dtype, prec):
     if dtype == torch.float64 and prec == "fp32_refine":
         compare(sb, got, obj_rtol=1e-8)
     assert solver.sync_error() == 0
+
+
+# LPs that would share a warp (two of up to 15, one of up to 31 rows and columns), enough of
+# them to leave the kernel that does so.
+@pytest.mark.parametrize("m,n", [(8, 1), (1, 8), (9, 15), (15, 15), (16, 16), (1, 31), (31, 1), (20, 27), (31, 31)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_same_pivots_as_several_lps_per_warp(solver, m, n, dtype):
+    sb = synth.type1(20001, m, n, seed=m + 1000 * n)
+    batch = _batch(sb, dtype)
+    got, ref = host(solver.solve(batch, prec="fp32")), host(solver.solve(batch, prec="fp32", kernel=PACK))
+    for name in ("status", "iters", "basis", "obj", "x", "y"):
+        assert np.array_equal(got[name], ref[name]), name
 
 
 @pytest.mark.parametrize("m,n", [(40, 33), (64, 64), (130, 30)])
