@@ -7,8 +7,8 @@ refinement and KKT certificate, FP64 re-solve of failures, outputs.  Prints one 
 
 Secondary legs (skip with ``--no-legs``) time the other workloads once each with CUDA
 events: 1,000 x m=n=16; the m=n sweep (5, 7, 12, 15 and 28 at 100,000 LPs: several tiny
-LPs per warp up to 15; 50 and 64: one warp per LP, the tableau in shared memory); the two Step 1 rules (most negative reduced cost vs a random
-eligible column) and steepest edge on 50,000 x m=n=100; one m=n=100 polytope in 50,000
+LPs per warp up to 15; 50 and 64: the kernel that keeps the pivots); the two Step 1 rules (most
+negative reduced cost vs a random eligible column) and steepest edge on 50,000 x m=n=100; one m=n=100 polytope in 50,000
 directions (shared constraints); 10,000 x m=n=100 with bounds l <= x <= u; 10,000 x m=n=200
 two-phase (largest coefficient and steepest edge); hyperbox support functions (4,000,000 x 5
 FP32, 6,000,000 x 28 FP64); 20,000 mixed sizes forward and forward+backward.
@@ -42,11 +42,11 @@ METRIC = "LPs/sec at m=n=100 (FP32+FP64-refine vs plain FP64, rel obj err<=1e-8)
 WORKLOAD = "type-1 LPs, 50,000 per GPU, m=n=100, A~U[0.1,1], b~U[1,10], c~U[0,1], seed 1"
 FP32_FMA_PIPES_PER_SM = 128
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per 50,000-LP launch of the
-# one-warp-per-LP kernel (the planner's choice at m = n = 100), from an ncu capture of a
+# kernel that keeps the pivots (the planner's choice at m = n = 100), from an ncu capture of a
 # 20,000-LP launch scaled by 2.5 (DRAM bytes grow with the LPs processed), keyed by the first
 # 16 hex digits of the sha256 of the kernel source it was taken on; a source without an entry
 # reports traffic null.
-PROFILED_DRAM_BYTES = {"9a92a40bc8d895a9": 4838.3e6}
+PROFILED_DRAM_BYTES = {"bc6bf48866951563": 5670.0e6}
 
 
 def parse():
@@ -167,7 +167,7 @@ class ClockSampler:
 
 
 def kernel_source_hash() -> str:
-    src = open(os.path.join(ROOT, "paper_1609_08114_gb300", "csrc", "simplex_warp.cu"), "rb").read()
+    src = open(os.path.join(ROOT, "paper_1609_08114_gb300", "csrc", "simplex_lazy.cuh"), "rb").read()
     return hashlib.sha256(src).hexdigest()[:16]
 
 

@@ -113,11 +113,15 @@ typedef struct {
   int32_t reg_warps;         /* warps per LP of the register kernel: 1 (m, n <= 31), 4 or 8
                                 [autotuned, else 1 when every LP has m, n <= 31, else 8; with
                                 kernel = AUTO and reg_warps = 0, batches of LPs with m, n <= 31
-                                take the several-LPs-per-warp kernel (LPB_KERNEL_PACK), and
-                                FP64-input batches (or size classes) with 32 <= max(m, n) take
-                                LPB_KERNEL_WARP up to m n = 10000, and beyond that where an SM
-                                holds four of its LPs (with refinement: while one register-kernel
-                                CTA per SM fits)] */
+                                in an FP32 mode take the several-LPs-per-warp kernel
+                                (LPB_KERNEL_PACK; many of them in plain FP32 another kernel
+                                with the same results); other LPs with b >= 0 take, under the
+                                largest coefficient rule and mostly under the random rule, the kernel
+                                that keeps the pivots instead of a tableau, in the arithmetic of
+                                the kernel that an FP64-input batch (or size class) with 32 <=
+                                max(m, n) would otherwise take: LPB_KERNEL_WARP up to m n =
+                                10000, and beyond that where an SM holds four of its LPs (with
+                                refinement: while one register-kernel CTA per SM fits)] */
   int32_t pivot_rule;        /* lpb_pivot_rule: Step 1's entering-column rule [LPB_PIVOT_LPC] */
   uint64_t seed;             /* LPB_PIVOT_RPC: seed of the counter-based random draw [0] */
 } lpb_options;
@@ -168,7 +172,10 @@ lpb_err lpb_destroy(lpb_handle *handle);
 /* Workspace bytes lpb_solve / lpb_solve_backward need for this batch shape
  * and these options (depends only on count, max_m, max_n, min_m, min_n,
  * dtype and the options; a solve whose batch declares other sizes than the
- * query may need more and then returns LPB_ENOMEM before any launch). */
+ * query may need more and then returns LPB_ENOMEM before any launch).  Part
+ * of it holds pivots that the automatic kernels keep; a solve that gets a
+ * workspace without room for those, but enough for the kernels that update the
+ * whole tableau, runs on these, with the same results, slower. */
 lpb_err lpb_workspace_size(lpb_handle *handle, const lpb_batch *batch, const lpb_options *opt,
                            size_t *bytes);
 
@@ -202,7 +209,7 @@ lpb_err lpb_hyperbox(lpb_handle *handle, int64_t count, int32_t n, int32_t dtype
                      void *obj, void *x, void *stream);
 
 /* Autotuner.  Picks, for batches shaped like `batch` (same max_m, max_n,
- * dtype and precision), the fastest schedule among: warps per LP of the
+ * dtype and precision), the fastest schedule among: the default, warps per LP of the
  * register kernel (1, 4 or 8), the one-warp-per-LP shared-memory kernel
  * (LPB_KERNEL_WARP, where it applies), threads per CTA of the tableau kernel
  * (automatic, 256, 512 or 1024) and its placement (shared memory when it
