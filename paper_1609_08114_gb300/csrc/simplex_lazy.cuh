@@ -894,6 +894,8 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         if ((!fail && !more) || round == 2) break;
       }
     }
+    // The corrected values of other lanes are read below (several warps: the vote's barrier).
+    if constexpr (W == 1) __syncwarp();
     if (!fail) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
