@@ -98,13 +98,14 @@ template <typename T> using Img = std::conditional_t<sizeof(T) == 8, unsigned lo
 // conversion runs on the slow FP64 unit).
 __device__ __forceinline__ double widen(double v) { return v; }
 __device__ __forceinline__ double widen(float v) { return f2d_exact(v); }
-// The same for a finite entry of A in the FP64 products, without branches:
-// magnitudes below the smallest normal float count as zero.
-__device__ __forceinline__ double widen_a(double v) { return v; }
-__device__ __forceinline__ double widen_a(float v) {
+// The same for a zero or normal entry of A in the FP64 products, without
+// branches; `low`: the least magnitude image minus one, by which the caller
+// finds the subnormal ones.
+__device__ __forceinline__ double widen_a(double v, unsigned &) { return v; }
+__device__ __forceinline__ double widen_a(float v, unsigned &low) {
   const unsigned u = __float_as_uint(v), mag = u & 0x7fffffffu;
-  const bool z = mag < 0x00800000u;
-  return __hiloint2double(int((u & 0x80000000u) | (z ? 0u : (mag >> 3) + (896u << 20))), int(z ? 0u : u << 29));
+  low = min(low, mag - 1u);
+  return __hiloint2double(int((u & 0x80000000u) | (mag == 0u ? 0u : (mag >> 3) + (896u << 20))), int(u << 29));
 }
 
 // Entry `i` of the LP's A as the tableau's type: RN = false truncates FP64 to
@@ -763,9 +764,10 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       for (int round = 0;; ++round) {
         sync();
         // b - A x by row and A^T y - c by column, in FP64.
-        double sx[R], sy[R];
+        double ra[R], rd[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) sx[r] = sy[r] = 0.0;
+        for (int r = 0; r < R; ++r) ra[r] = rd[r] = 0.0;
+        unsigned low = 0xffffffffu;
 #pragma unroll 1
         for (int q = 0; q < k; q += 4) {
           In va[4][R], vb[4][R];
@@ -784,92 +786,135 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
               const double x = xq[q + u], y = xq[kx + q + u];
 #pragma unroll
               for (int r = 0; r < R; ++r) {
-                sx[r] = fma(widen_a(va[u][r]), x, sx[r]);
-                sy[r] = fma(widen_a(vb[u][r]), y, sy[r]);
+                ra[r] = fma(widen_a(va[u][r], low), x, ra[r]);
+                rd[r] = fma(widen_a(vb[u][r], low), y, rd[r]);
               }
             }
         }
+        if (!F64 && low < 0x007fffffu) {     // subnormal entries: again, by the hardware's conversion
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            ra[r] = rd[r] = 0.0;
+#pragma unroll 1
+            for (int q = 0; q < k; ++q) {
+              ra[r] = fma(double(__ldg(A + (ic[r] * n + off[q]))), xq[q], ra[r]);
+              rd[r] = fma(double(__ldg(A + (off[kx + q] + jc[r]))), xq[kx + q], rd[r]);
+            }
+          }
+        }
         // The residuals that a correction has to take up are those of the binding
         // rows and of the basic structurals' columns (a basic slack takes its own).
-        float rp_[R], rd_[R], v[R], w[R];
+        float v[R], w[R], rp_[R], rd_[R];
+        int more = 0;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          rp_[r] = __double2float_rn(widen(__ldg(bg + ic[r])) - sx[r]);
-          rd_[r] = __double2float_rn(sy[r] - widen(__ldg(cg + jc[r])));
-          v[r] = in_m[r] && flag[tid + NT * r] ? rp_[r] : 0.f;
-          w[r] = in_n[r] && flag[D + tid + NT * r] ? rd_[r] : 0.f;
+          ra[r] = widen(__ldg(bg + ic[r])) - ra[r];
+          rd[r] = rd[r] - widen(__ldg(cg + jc[r]));
+          const bool tr = in_m[r] && flag[tid + NT * r], tc = in_n[r] && flag[D + tid + NT * r];
+          v[r] = __double2float_rn(ra[r]);
+          w[r] = __double2float_rn(rd[r]);
+          if constexpr (!RN) { rp_[r] = v[r]; rd_[r] = w[r]; }
+          v[r] = tr ? v[r] : 0.f;
+          w[r] = tc ? w[r] : 0.f;
+          // RN: as the tableau kernel does, corrections (three at most) until the
+          // residuals are far below the certificate's bar: 4000 times, because that
+          // kernel asks for 1000 times in the rows of basic slacks too.  (Largest
+          // error in x against FP64, 99% quantile over 10,000 bounded LPs of 100 x
+          // 100: tableau kernel 2.2e-11, here 2.5e-11 with 1000 times.)
+          if constexpr (RN)
+            more |= int(tr && !dge(0.25e-3 * tp, abs_bits(ra[r]))) | int(tc && !dge(0.25e-3 * td, abs_bits(rd[r])));
         }
-        // Corrections with the FP32 basis inverse: the pivots on v as another
-        // right-hand side, on w as another objective row.
-        through_pivots(v, w);
+        bool correct = true;
+        if constexpr (RN) correct = any(more) && round < 3;
+        if (correct) {
+          // Corrections with the FP32 basis inverse: the pivots on v as another
+          // right-hand side, on w as another objective row.
+          through_pivots(v, w);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (qi[r] >= 0) dv[qi[r]] = v[r];
-          if (pi[r] >= 0) dv[kx + pi[r]] = w[r];
+          for (int r = 0; r < R; ++r) {
+            if (qi[r] >= 0) dv[qi[r]] = v[r];
+            if (pi[r] >= 0) dv[kx + pi[r]] = w[r];
+          }
+          sync();
         }
-        sync();
         // The corrected x and y, and c^T x and b^T y.
         int bd = 0;
         double cxp = 0.0, byp = 0.0, by;
 #pragma unroll 1
         for (int q = tid; q < k; q += NT) {
-          const double x = xq[q] + widen(dv[q]), y = xq[kx + q] + widen(dv[kx + q]);
-          xq[q] = x;
-          xq[kx + q] = y;
+          double x = xq[q], y = xq[kx + q];
+          if (correct) {
+            x += widen(dv[q]);
+            y += widen(dv[kx + q]);
+            xq[q] = x;
+            xq[kx + q] = y;
+          }
           bd |= int(!dge(x, neg_bits(tp))) | int(!dge(y, neg_bits(td)));
           cxp = fma(widen(__ldg(cg + off[q])), x, cxp);
           byp = fma(widen(__ldg(bg + kr[q])), y, byp);
         }
         // KKT certificate of the pair that is written out: x >= 0, A x <= b,
         // y >= 0, A^T y >= c and c^T x = b^T y, each to tol scaled by the data.
-        // b - A x and A^T y - c at the corrected point are the residuals (rounded
-        // to FP32 here) plus FP32 products with the corrections; their rounding
-        // (and the 2^-20 truncation of A) is bounded by 2^-15 times the sum of the
-        // products' magnitudes and 2^-22 of the residual.
-        float dl[R], mg[R], el[R], eg[R];
+        // RN: on the residuals of that pair.  Else b - A x and A^T y - c at the
+        // corrected point are the FP64 residuals plus FP32 products with the
+        // corrections; their rounding (m, n <= 127 terms, and the 2^-20 truncation
+        // of A) is bounded by 2^-15 times the sum of the products' magnitudes.
+        if constexpr (RN) {
+          if (correct) continue;
 #pragma unroll
-        for (int r = 0; r < R; ++r) dl[r] = mg[r] = el[r] = eg[r] = 0.f;
+          for (int r = 0; r < R; ++r)
+            bd |= int(in_m[r] && !dge(ra[r], neg_bits(tp))) | int(in_n[r] && !dge(rd[r], neg_bits(td)));
+        } else {
+          float dl[R], mg[R], el[R], eg[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) dl[r] = mg[r] = el[r] = eg[r] = 0.f;
 #pragma unroll 1
-        for (int q = 0; q < k; q += 4) {
-          unsigned va[4][R], vb[4][R];
-          const unsigned *Aw = reinterpret_cast<const unsigned *>(A);
-          constexpr int es = sizeof(In) / 4;
+          for (int q = 0; q < k; q += 4) {
+            unsigned va[4][R], vb[4][R];
+            const unsigned *Aw = reinterpret_cast<const unsigned *>(A);
+            constexpr int es = sizeof(In) / 4;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int j = off[q + u], i = off[kx + q + u];
+            for (int u = 0; u < 4; ++u) {
+              const int j = off[q + u], i = off[kx + q + u];
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-              va[u][r] = __ldg(Aw + es * (ic[r] * n + j) + es - 1);
-              vb[u][r] = __ldg(Aw + es * (i + jc[r]) + es - 1);
+              for (int r = 0; r < R; ++r) {
+                va[u][r] = __ldg(Aw + es * (ic[r] * n + j) + es - 1);
+                vb[u][r] = __ldg(Aw + es * (i + jc[r]) + es - 1);
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const float d = dv[q + u], g = dv[kx + q + u];
+#pragma unroll
+              for (int r = 0; r < R; ++r) {
+                const float a = F64 ? hi2f(va[u][r]) : __uint_as_float(va[u][r]);
+                const float b = F64 ? hi2f(vb[u][r]) : __uint_as_float(vb[u][r]);
+                dl[r] = fmaf(a, d, dl[r]);
+                mg[r] = fmaf(fabsf(a), fabsf(d), mg[r]);
+                el[r] = fmaf(b, g, el[r]);
+                eg[r] = fmaf(fabsf(b), fabsf(g), eg[r]);
+              }
             }
           }
+          // In FP32 first, with 2^-22 of the residual for its rounding; what does not
+          // pass there is compared in FP64.
+          const float lim_p = -__double2float_rd(tp), lim_d = -__double2float_rd(td);
+          int near_bar = 0;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float d = dv[q + u], g = dv[kx + q + u];
+          for (int r = 0; r < R; ++r) {
+            const float rp = rp_[r], rq = rd_[r];
+            const float sp = rp - dl[r] - fmaf(kDeltaErr, mg[r], 0x1p-22f * fabsf(rp));
+            const float sd = rq + el[r] - fmaf(kDeltaErr, eg[r], 0x1p-22f * fabsf(rq));
+            near_bar |= int(in_m[r] && !(sp >= lim_p)) | int(in_n[r] && !(sd >= lim_d));
+          }
+          if (near_bar) {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-              const float a = F64 ? hi2f(va[u][r]) : __uint_as_float(va[u][r]);
-              const float b = F64 ? hi2f(vb[u][r]) : __uint_as_float(vb[u][r]);
-              dl[r] = fmaf(a, d, dl[r]);
-              mg[r] = fmaf(fabsf(a), fabsf(d), mg[r]);
-              el[r] = fmaf(b, g, el[r]);
-              eg[r] = fmaf(fabsf(b), fabsf(g), eg[r]);
+              const double sp = ra[r] - widen(fmaf(kDeltaErr, mg[r], dl[r]));
+              const double sd = rd[r] + widen(fmaf(-kDeltaErr, eg[r], el[r]));
+              bd |= int(in_m[r] && !dge(sp, neg_bits(tp))) | int(in_n[r] && !dge(sd, neg_bits(td)));
             }
           }
-        }
-        const float lim_p = -__double2float_rd(tp), lim_d = -__double2float_rd(td);
-        int more = 0;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const float np = rp_[r] - dl[r], nd = rd_[r] + el[r];
-          const float sp = np - fmaf(kDeltaErr, mg[r], 0x1p-22f * fabsf(rp_[r]));
-          const float sd = nd - fmaf(kDeltaErr, eg[r], 0x1p-22f * fabsf(rd_[r]));
-          // RN: as the tableau kernel does, another correction while the
-          // residuals left are not 1000 times below the certificate's bar.
-          if constexpr (RN)
-            more |= int(in_m[r] && flag[tid + NT * r] && fabsf(np) > -1e-3f * lim_p) |
-                    int(in_n[r] && flag[D + tid + NT * r] && fabsf(nd) > -1e-3f * lim_d);
-          bd |= int(in_m[r] && !(sp >= lim_p)) | int(in_n[r] && !(sd >= lim_d));
         }
         if constexpr (W == 1) {
           cx = warp_sum(cxp);
@@ -890,8 +935,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         }
         bd |= !(fabs(cx - by) <= tol * (1.0 + fabs(cx)));
         fail = any(bd);
-        if constexpr (RN) more = any(more);
-        if ((!fail && !more) || round == 2) break;
+        if (RN || !fail || round == 2) break;
       }
     }
     // The corrected values of other lanes are read below (several warps: the vote's barrier).
