@@ -290,8 +290,8 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // 0.13; 10,000 x 28 0.099 -> 0.052), from as many LPs on as take longer than the
 // host takes to plan and launch (10,000 x 12 0.048 and 0.050, 1,000 x 30 x 20
 // 0.047 and 0.049).  With four (m, n <= 7) that kernel's lanes are full.  Its refinement corrects by products with the final
-// tableau, which this kernel does not have: another rounding of the results, so
-// refined passes stay.
+// tableau, which this kernel mostly does not have: another rounding of the results,
+// so refined passes stay.
 // The random rule takes over three times the pivots (45.6 against 13.3 at
 // 100 x 100), so its chains are longer and a full update is the better one in
 // places: it comes here only with enough LPs to fill the GPU (300 x 100 FP64 0.98
@@ -306,10 +306,18 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // 2.38 ms with 8, 2.18 with 12, 2.12 with 16, 2.18 with 20; 2,000 x 300: 2.37
 // with 16, 2.06 with 30, 3.16 with 48).  FP64 entries are twice as large and its
 // chains are bound by the FP64 pipe, so fewer pay (20,000 x 100: 1.38 with 8,
-// 1.53 with 12).  At most kmax pivots: an LP beyond it starts again in the
-// tableau kernel, so it lies above what LPs with a bound on every variable take
-// (200 x 100, 64 pivots on average, 100 at most: 10,000 in 9.5 ms with none
-// handed on, 16 ms with 45% handed on, 17.5 ms all by the tableau kernel).
+// 1.53 with 12).
+// Pivots kept before they are applied to a tableau in the slot: as many as type-1
+// LPs take at most (39 of 50,000 at 100 x 100, 30 at 64 x 64, 22 at 48 x 37, 69 at
+// 300 x 300: about 4 sqrt(min(m, n)); under the random rule two to four times
+// that), which an application would cost more than the chains.  LPs of many pivots
+// would have it earlier, as the entries beyond the shared ones come from L2 (20,000 x
+// 100 x 100, normal rows, 126 pivots, plain FP32: 9.5 ms with 27, 9.9 with 34, 10.2
+// with 37, where 50,000 type-1 LPs take 2.25, 2.13, 2.14).  FP64: 58 ms with 42, 63
+// with 58 (type-1 1.6 ms with 32, 1.37 with 42).  Four and eight warps per LP: 4,000 x
+// 200 x 100 with one entry in ten, 102 pivots, 4.2 ms with 42, 5.0 with 72, 5.4 with
+// 100; 10,000 LPs with a bound on every variable, 64 pivots, 9.2, 8.2, 7.9.  The
+// kernels that update the whole tableau: 8.6 (plain FP32), 101 (FP64), 10.0 and 17.7 ms.
 void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int shared, Pass *p) {
   if ((o->kernel != LPB_KERNEL_AUTO && shared != 2) || o->threads != 0 || o->reg_warps != 0) return;
   if (o->pivot_rule == LPB_PIVOT_STEEPEST) return;
@@ -328,10 +336,14 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
     if (p->warp || b->count < 16 * d.sms) return;
     if (kind == LAZY_FP64 ? mx > 8 * mn : kind == LAZY_SMALL ? mx > 64 : q.max_n > 128) return;
   }
-  q.kmax = (64 + (rpc ? mn : mn / 2) + 3) & ~3;
+  const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 ? 4 : 3.25) * (!rpc ? 1 : kind == LAZY_FP64 ? 4 : 2);
+  q.kmax = 2 + int(keep * std::sqrt(double(mn)));
   q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL || kind == LAZY_PACK ? 6 + mn / 10 : 8 + mn / 4;
   const int most = 72 * 1024 / ((q.max_m + q.max_n) * eb);      // a third of an SM's shared memory
-  if (q.ks > most) q.ks = most > 1 ? most : 1;
+  if (q.ks > most) q.ks = most;
+  if (q.ks < 2) q.ks = 2;
+  if (q.kmax < q.ks) q.kmax = q.ks;
+  q.kw = q.ks;
   int occ = 0, threads = 0;
   LazyLayout lay{};
   const cudaError_t ce = kLazyOccupancy[rpc][kind](q, b->dtype, &occ, &threads, &lay);
@@ -342,14 +354,14 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
   p->lay = lay;
   p->threads = threads;
   p->smem = size_t(lay.bytes);
-  p->slot_bytes = (size_t(q.kmax - q.ks) * lay.hs * eb + 127) & ~size_t(127);
+  p->slot_bytes = ((size_t(q.kmax - q.ks) * lay.hs + size_t(q.max_m) * lay.ld) * eb + 127) & ~size_t(127);
   p->gmem = true;
   p->grid = occ * d.sms;
   if (p->grid > b->count) p->grid = b->count > 0 ? b->count : 1;
 }
 
-// `plain`: full updates after every pivot in every pass (no history slots, more
-// rows in shared memory).
+// `plain`: full updates after every pivot in every pass (no history and tableau
+// slots, more rows in shared memory).
 lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, bool basis_given,
                   Plan *pl, bool plain = false, int shared = 0) {
   if (!b || !o) return LPB_EINVAL;

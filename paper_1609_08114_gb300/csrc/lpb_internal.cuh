@@ -441,12 +441,15 @@ int warp_tab_bytes(int max_m, int max_n);
 // fp64: FP64.
 struct LazyShape {
   int max_m, max_n;
-  int ks, kmax;                // history entries in shared memory; pivots at most
+  int ks;                      // history entries in shared memory (two at least)
+  int kmax, kw;                // pivots kept before they are applied: the first time, later
   bool shared;                 // objectives of one polytope
 };
 struct LazyLayout {
-  int hs;                      // elements of a history entry
-  int ks, kmax;
+  int hs, pn;                  // elements of a history entry, and where its pivot row starts
+  int ks, kmax, kw;
+  int kx;                      // basic structurals at most
+  int ld;                      // row stride of the slot's tableau
   int tab;                     // > 0: the warp kernel's limit on basic structurals, from these bytes
   int hist, rp, at, xq, dv, off, kr, flag, red;   // byte offsets
   int bytes;

@@ -21,14 +21,21 @@
 //   * History entry s holds f_s (m values) and p_s (n values), with f_s[l] =
 //     -1/p and p_s[e] = 1, so that one multiply-add from -0 restarts a chain.
 //     The first `ks` entries live in shared memory, the rest (few LPs take that
-//     many pivots) in a slot of the workspace; an LP of more than `kmax` pivots
-//     goes to the tableau kernel, whose pivots cost the same at any number.
+//     many pivots) in a slot of the workspace.
+//   * An LP of more than `kmax` pivots (the planner's rule, by size) has a tableau after
+//     all: the history is applied to A in one pass, into the slot, and later to
+//     that tableau, whenever `ks` more pivots are kept.  The chains then start from the
+//     slot's entries.  The order of operations on an entry is the same, so are the
+//     values.  (20,000 x 100 x 100 with normal rows, 126 pivots: FP64 134 ms when such
+//     LPs started again in the tableau kernel, 58 now, 101 with a full update per pivot;
+//     plain FP32 28.9, 9.9 and 8.6.)
 //   * A is read where it lies: one pass over it checks that it is finite (and
 //     leaves it in L2), then a pivot reads the one row and column it needs.
 //   * Refinement and certificate (FP32 + refinement): FP64 residuals from A; the
 //     correction B^-1 r by running the pivots on r as another right-hand side,
-//     its transpose as another objective row (k (m + n) operations); the KKT
-//     certificate of the other kernels.
+//     its transpose as another objective row (k (m + n) operations), or by products
+//     with the slot's tableau where there is one; the KKT certificate of the other
+//     kernels.
 //   * Objectives of one polytope (lpb_solve_shared): a CTA takes consecutive ones
 //     and starts each from the basis of the one before, whose history, right-hand
 //     side and variables it keeps: the new objective row is -c run through the
@@ -57,6 +64,15 @@ namespace {
 // between two cold ones.
 constexpr int kShareChunk = 16;
 constexpr int kWarmMax = 32;
+// Rows of a column that a thread takes at a time when pivots are applied (the
+// history's pivot rows start at a multiple of it).
+constexpr int kApplyRows = 8;
+// Residuals, in parts of the certificate's bar, at which refinement stops (the tableau
+// kernel's arithmetic): a quarter of that kernel's, which asks for it in the rows of
+// basic slacks too.  (Error in x against FP64, 99% quantile over 10,000 bounded LPs of
+// 100 x 100: tableau kernel 2.2e-11; here 2.5e-11 with its 1e-3, 1.2e-11 with this.)
+constexpr double kStop = 0.25e-3;
+constexpr int kApplyCols = 2;
 enum : int { kCommon = 0, kShared = 1, kRandom = 2, kPacked = 3 };
 
 __device__ __forceinline__ float neg(float v) { return -v; }
@@ -159,6 +175,52 @@ __device__ __forceinline__ unsigned scan_a(const void *A, int cnt, int tid) {
   return amax;
 }
 
+// kApplyRows values of one column and the multiply-add of a pivot on them, x <- x - f p.
+// FP32 in pairs: one fma.rn.f32x2 rounds its halves as two fmaf do.
+template <typename T> struct Rows;
+template <>
+struct Rows<float> {
+  unsigned long long v[kApplyRows / 2];
+  static __device__ __forceinline__ unsigned long long pair(float a, float b) {
+    return (static_cast<unsigned long long>(__float_as_uint(b)) << 32) | __float_as_uint(a);
+  }
+  __device__ __forceinline__ void load(const float *p) {           // at a 16-byte boundary
+#pragma unroll
+    for (int u = 0; u < kApplyRows / 4; ++u) {
+      const ulonglong2 a = reinterpret_cast<const ulonglong2 *>(p)[u];
+      v[2 * u] = a.x;
+      v[2 * u + 1] = a.y;
+    }
+  }
+  __device__ __forceinline__ float get(int u) const { return __uint_as_float(unsigned(u & 1 ? v[u / 2] >> 32 : v[u / 2])); }
+  __device__ __forceinline__ void set(int u, float x) {
+    v[u / 2] = u & 1 ? pair(__uint_as_float(unsigned(v[u / 2])), x) : pair(x, __uint_as_float(unsigned(v[u / 2] >> 32)));
+  }
+  __device__ __forceinline__ void sub(const Rows &f, float p) {
+    const unsigned long long q = pair(-p, -p);
+#pragma unroll
+    for (int u = 0; u < kApplyRows / 2; ++u) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v[u]) : "l"(f.v[u]), "l"(q));
+  }
+};
+template <>
+struct Rows<double> {
+  double v[kApplyRows];
+  __device__ __forceinline__ void load(const double *p) {
+#pragma unroll
+    for (int u = 0; u < kApplyRows / 2; ++u) {
+      const double2 a = reinterpret_cast<const double2 *>(p)[u];
+      v[2 * u] = a.x;
+      v[2 * u + 1] = a.y;
+    }
+  }
+  __device__ __forceinline__ double get(int u) const { return v[u]; }
+  __device__ __forceinline__ void set(int u, double x) { v[u] = x; }
+  __device__ __forceinline__ void sub(const Rows &f, double p) {
+#pragma unroll
+    for (int u = 0; u < kApplyRows; ++u) v[u] = fma(neg_bits(f.v[u]), p, v[u]);
+  }
+};
+
 // Full-precision reciprocal (correctly rounded, the value of 1 / x).
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
@@ -175,26 +237,192 @@ struct __align__(16) Cand {
 
 // Shared memory of one CTA: `ks` history entries, then the small arrays.
 template <typename T>
-__host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warps, int rows, int ks, int kmax) {
+__host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warps, int rows, int ks, int kmax, int kw) {
   LazyLayout L{};
-  L.hs = lim_m + lim_n;
+  L.pn = (lim_m + kApplyRows - 1) & ~(kApplyRows - 1);
+  L.hs = L.pn + ((lim_n + 3) & ~3);
   L.ks = ks;
   L.kmax = kmax;
+  L.kw = kw;
+  L.ld = lim_n;
+  L.kx = ((lim_m < lim_n ? lim_m : lim_n) + 3) & ~3;
   int o = 0;
   auto take = [&](int bytes) { const int at = o; o = (o + bytes + 15) & ~15; return at; };
   L.hist = take(ks * L.hs * int(sizeof(T)));
   L.rp = take(kmax * int(sizeof(T)));
   L.at = take(kmax * 4);
   if (sizeof(T) == 4) {
-    L.xq = take(2 * kmax * 8);
-    L.dv = take(2 * kmax * 4);
-    L.off = take(2 * kmax * 4);
-    L.kr = take(kmax * 2);
+    L.xq = take(2 * L.kx * 8);
+    L.dv = take(2 * L.kx * 4);
+    L.off = take(2 * L.kx * 4);
+    L.kr = take(L.kx * 2);
     L.flag = take(2 * 32 * warps * rows);
   }
   L.red = take(warps > 1 ? 2 * warps * int(sizeof(Cand<T>)) + 8 * warps * 8 + 16 : 0);
   L.bytes = o;
   return L;
+}
+
+// The pivots of the history on the tableau in the slot (`based`; else on A), into the
+// slot: kApplyRows rows of kApplyCols columns (FP64: of one) per thread at a time, with
+// every pivot before they are stored, so that one pass over the tableau serves all of
+// them.  Bound by the latency of that pass with a few warps per LP: two columns halve the
+// round trips to L2 (20,000 x 100 x 100 of 126 pivots, plain FP32, inlined: 10.1 ms with one,
+// 9.1 with two, 8.8 with four, which take registers from the kernel).  Not inlined, and
+// called outside of the pivot loop: LPs of few pivots never get here, and its code cost
+// them 4% (50,000 x 100) to 15% (48 x 37) there.
+template <typename T, int NT, bool F64, bool RN>
+__device__ __noinline__ void apply_pivots(T *tab, const T *spill, const void *A, int m, int n, int held, bool based,
+                                          int hist_at, int ats_at, int ks, int hs, int pn, int ld) {
+  extern __shared__ __align__(16) unsigned char lz_smem[];
+  __builtin_assume(__isGlobal(tab));
+  __builtin_assume(__isGlobal(spill));
+  __builtin_assume(__isGlobal(A));
+  constexpr int NC = sizeof(T) == 8 ? 1 : kApplyCols;
+  const T *hist = reinterpret_cast<const T *>(lz_smem + hist_at);
+  const unsigned *ats = reinterpret_cast<const unsigned *>(lz_smem + ats_at);
+  const int nj = (n + NC - 1) / NC, tasks = (m + kApplyRows - 1) / kApplyRows * nj;
+#pragma unroll 1
+  for (int t = threadIdx.x; t < tasks; t += NT) {
+    const int ib = t / nj, j0 = t - ib * nj, i0 = ib * kApplyRows;
+    int j[NC];                 // (past the end: the last column, not stored)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) j[c] = min(j0 + c * nj, n - 1);
+    Rows<T> x[NC];
+#pragma unroll
+    for (int u = 0; u < kApplyRows; ++u) {
+      const int i = min(i0 + u, m - 1);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) x[c].set(u, based ? tab[i * ld + j[c]] : a_in<T, F64, RN>(A, i * n + j[c]));
+    }
+    auto steps = [&](auto U, const T *first, int s0, int s1) {
+#pragma unroll U.value
+      for (int s = s0; s < s1; ++s) {
+        const T *h = first + (s - s0) * hs;
+        Rows<T> f;
+        T p[NC];
+        f.load(h + i0);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) p[c] = h[pn + j[c]];
+        const int l = int(ats[s] >> 16) - i0, e = int(ats[s] & 0xffffu);
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+          if (j[c] == e) {
+#pragma unroll
+            for (int u = 0; u < kApplyRows; ++u) x[c].set(u, neg_zero<T>());
+          }
+        if (unsigned(l) < unsigned(kApplyRows)) {
+#pragma unroll
+          for (int u = 0; u < kApplyRows; ++u)
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+              if (u == l) x[c].set(u, neg_zero<T>());
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) x[c].sub(f, p[c]);
+      }
+    };
+    steps(std::integral_constant<int, 2>(), hist, 0, held < ks ? held : ks);
+    steps(std::integral_constant<int, sizeof(T) == 8 ? 2 : 4>(), spill, ks, held);
+#pragma unroll
+    for (int u = 0; u < kApplyRows; ++u)
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        if (i0 + u < m && j0 + c * nj < n) tab[(i0 + u) * ld + j[c]] = x[c].get(u);
+  }
+}
+
+// Refinement and certificate of an LP whose tableau is in the slot: as the tableau kernel
+// does, at most three corrections, by products with the tableau's rows of basic
+// structurals and columns of non-basic slacks, until the FP64 residuals are far below the
+// certificate's bar, which they are then held against.  x and y in `xq`; returns c^T x, NaN
+// where the certificate fails.
+template <int W, bool F64>
+__device__ __noinline__ double refine_by_tableau(const float *tab, const void *A_, const void *b_, const void *c_, int m,
+                                                 int n, int ld, int k, int kx, int hist_at, int hs, int pn, int xq_at,
+                                                 int off_at, int kr_at, int flag_at, int rows_at, int sums_at, double tol,
+                                                 double tp, double td) {
+  extern __shared__ __align__(16) unsigned char lz_smem[];
+  __builtin_assume(__isGlobal(tab));
+  __builtin_assume(__isGlobal(A_));
+  __builtin_assume(__isGlobal(b_));
+  __builtin_assume(__isGlobal(c_));
+  using In = std::conditional_t<F64, double, float>;
+  constexpr int NT = 32 * W;
+  const In *A = static_cast<const In *>(A_), *b = static_cast<const In *>(b_), *c = static_cast<const In *>(c_);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  float *res = reinterpret_cast<float *>(lz_smem + hist_at);         // residuals by row, and by column from pn on
+  const short *cp = reinterpret_cast<const short *>(res + hs), *rq = cp + kx;
+  double *xq = reinterpret_cast<double *>(lz_smem + xq_at), *sums = reinterpret_cast<double *>(lz_smem + sums_at);
+  const int *off = reinterpret_cast<const int *>(lz_smem + off_at);
+  const short *kr = reinterpret_cast<const short *>(lz_smem + kr_at);
+  const unsigned char *row_in = lz_smem + flag_at, *col_in = lz_smem + rows_at;
+  auto any = [&](int v) -> int {
+    if constexpr (W == 1) return __any_sync(kFull, v);
+    else return __syncthreads_or(v);
+  };
+  int bd;
+#pragma unroll 1
+  for (int step = 0;; ++step) {
+    if constexpr (W == 1) __syncwarp();
+    else __syncthreads();
+    int more = 0;
+    bd = 0;
+#pragma unroll 1
+    for (int i = tid; i < m; i += NT) {
+      double s = 0.0;
+#pragma unroll 4
+      for (int q = 0; q < k; ++q) s = fma(double(__ldg(A + (i * n + off[q]))), xq[q], s);
+      const double r = double(__ldg(b + i)) - s;
+      res[i] = __double2float_rn(r);
+      bd |= !(r >= -tp);
+      more |= row_in[i] && !(fabs(r) <= kStop * tp);
+    }
+#pragma unroll 1
+    for (int j = tid; j < n; j += NT) {
+      double s = 0.0;
+#pragma unroll 4
+      for (int q = 0; q < k; ++q) s = fma(double(__ldg(A + (off[kx + q] + j))), xq[kx + q], s);
+      const double d = s - double(__ldg(c + j));
+      res[pn + j] = __double2float_rn(d);
+      bd |= !(d >= -td);
+      more |= col_in[j] && !(fabs(d) <= kStop * td);
+    }
+    if constexpr (W == 1) __syncwarp();      // (several warps: the vote's barrier)
+    if (!any(more) || step == 3) break;
+#pragma unroll 1
+    for (int t = tid; t < k; t += NT) {
+      const float *row = tab + rq[t] * ld, *column = tab + cp[t];
+      float dx = 0.f, dy = 0.f;
+#pragma unroll 4
+      for (int q = 0; q < k; ++q) {
+        dx = fmaf(row[cp[q]], res[kr[q]], dx);
+        dy = fmaf(-column[rq[q] * ld], res[pn + off[q]], dy);
+      }
+      xq[t] += double(dx);
+      xq[kx + t] += double(dy);
+    }
+  }
+  double cx = 0.0, by = 0.0;
+  for (int q = tid; q < k; q += NT) {
+    const double x = xq[q], y = xq[kx + q];
+    bd |= int(!(x >= -tp)) | int(!(y >= -td));
+    cx = fma(double(__ldg(c + off[q])), x, cx);
+    by = fma(double(__ldg(b + kr[q])), y, by);
+  }
+  cx = warp_sum(cx);
+  by = warp_sum(by);
+  if constexpr (W > 1) {
+    if (lane == 0) { sums[wid] = cx; sums[W + wid] = by; }
+    __syncthreads();
+    cx = by = 0.0;
+    for (int w = 0; w < W; ++w) {
+      cx += sums[w];
+      by += sums[W + w];
+    }
+  }
+  bd |= !(fabs(cx - by) <= tol * (1.0 + fabs(cx)));
+  return any(bd) ? __longlong_as_double(0x7ff8000000000000ll) : cx;
 }
 
 // T: the tableau's type; W warps and R rows (columns) per thread; F64: the
@@ -211,6 +439,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   using Im = Img<T>;
   constexpr int NT = 32 * W, D = NT * R;
   constexpr bool kD = sizeof(T) == 8, SHARED = KIND == kShared, PACKED = KIND == kPacked;
+  constexpr int kSpillUnroll = kD ? 1 : RN ? 4 : 2;    // history entries in flight from the workspace
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
   constexpr Im kNone = Im(~Im(0));
   T *hist = reinterpret_cast<T *>(lz_smem + L.hist);
@@ -223,10 +452,15 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   int *votes = reinterpret_cast<int *>(mags + 4 * W);
   float *fvote = reinterpret_cast<float *>(mags + 6 * W);
   int *claimed = reinterpret_cast<int *>(mags + 8 * W);
-  T *spill = P.slots ? reinterpret_cast<T *>(static_cast<unsigned char *>(P.slots) + size_t(blockIdx.x) * P.slot_bytes)
-                     : nullptr;
+  // The CTA's slot: history entries beyond `ks`, then the tableau of an LP of many pivots.
+  T *spill = reinterpret_cast<T *>(static_cast<unsigned char *>(P.slots) + size_t(blockIdx.x) * P.slot_bytes);
+  auto tableau = [&]() {           // (formed where it is needed: few LPs get there)
+    int entries = L.kmax - L.ks;
+    asm volatile("" : "+r"(entries));
+    return spill + size_t(entries) * size_t(L.hs);
+  };
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int hs = L.hs, ks = L.ks, pn = P.lim_m;
+  const int hs = L.hs, ks = L.ks, pn = L.pn;
   const int nitems = P.in.count ? min(*P.in.count, P.list_cap) : P.B.count;
   const T eps_p = T(P.eps_p), eps_d = T(P.eps_d);
 
@@ -286,6 +520,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   int rst[R], cst[R];              // last pivot on each row and column, -1: none
   unsigned long long bm = 0ull;    // largest |b| (its bits)
   int held = 0;                    // pivots in the history
+  bool based = false;              // they are pivots on the slot's tableau, not on A
   int warm_run = 0;                // objectives since a cold start; -1: the history is no basis of this polytope
   bool scanned = false;            // the shared A is known to be finite
   int cold_left = 0;               // objectives to start cold, since a warm start took many pivots
@@ -373,7 +608,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       item = nitem; lp = nlp; m = nm; n = nn; aoff = na; boff = nb; coff = nc;
       sync();
     };
-    auto defer = [&]() {           // the tableau kernel takes it (Phase I, sizes, bad data, many pivots)
+    auto defer = [&]() {           // the tableau kernel takes it (Phase I, sizes, bad data)
       if (tid == 0) {
         P.R.status[lp] = STATUS_PENDING;
         list_push(P.defer_items, P.defer_count, P.list_cap, lp, P.err);
@@ -389,7 +624,10 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       scanned = true;
       warm_run = warm ? warm_run + 1 : 0;
     }
-    if (!warm) held = 0;
+    if (!warm) {
+      held = 0;
+      based = false;
+    }
 
     // The block's best candidate: least image o[], then least key (kNone: no
     // candidate), with the values va, vb and the last pivot of its owner.  One
@@ -486,167 +724,192 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       sync();
       if constexpr (SHARED) through_pivots(nullptr, obj);
     }
-    bool bland = false, over = false;
+    bool bland = false;
 #pragma unroll 1
     for (;;) {
-      // Step 1: the most negative reduced cost (Bland: the lowest variable).
-      Im o[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        o[r] = in_n[r] && above(neg(obj[r]), eps_d) ? (bland ? Im(0) : image(obj[r])) : kNone;
-        // The random rule: the least key of the variable at this pivot (FP32: of
-        // its upper 31 bits, as the register kernel ranks; RN: of all but the one
-        // value that stands for no candidate).
-        if constexpr (KIND == kRandom)
-          if (o[r] != kNone && !bland) {
-            const unsigned key = rpc_key(P.seed, P.lp_base + lp, iters, int(nkey[r] >> kIdxBits));
-            o[r] = kD ? Im(key) : RN ? Im(min(key, 0xfffffffeu)) : Im(key >> 1);
-          }
-      }
-      const Cand<T> col = choose(0, o, nkey, obj, obj, cst);
-      if (col.o == kNone) break;
-      const int e = int(col.key) & kIdxMask, cse = col.last;
-      // Column e: from A or from the pivot that last stood on it, then the pivots since.
-      T a[R];
-      const int e1 = held < ks ? held : ks;
-      {
-        int s = cse + 1;
-        if (cse < 0) {
-#pragma unroll
-          for (int r = 0; r < R; ++r) a[r] = a_in<T, F64, RN>(A, ic[r] * n + e);
-        } else {
-          const T *h = entry(cse);
-#pragma unroll
-          for (int r = 0; r < R; ++r) a[r] = neg(h[ic[r]]);
-        }
-#pragma unroll 4
-        for (; s < e1; ++s) {
-          const T *h = hist + s * hs;
-          const T pe = h[pn + e];
-#pragma unroll
-          for (int r = 0; r < R; ++r) a[r] = mul_add(neg(h[ic[r]]), pe, s == rst[r] ? neg_zero<T>() : a[r]);
-        }
+      bool full = false;
 #pragma unroll 1
-        for (; s < held; ++s) {
-          const T *h = spill + (s - ks) * hs;
-          const T pe = h[pn + e];
-#pragma unroll
-          for (int r = 0; r < R; ++r) a[r] = mul_add(neg(h[ic[r]]), pe, s == rst[r] ? neg_zero<T>() : a[r]);
-        }
-      }
-      // Step 2: the min-ratio test.
-      if constexpr (kD) {
-        // The ratios in FP32 first (relative error below 3e-7; FP64 division is
-        // slow here): only rows within 1e-5 of the smallest get the exact
-        // quotient, and none does when a single row is left whose ratio is
-        // clearly above the degeneracy threshold.
-        float q[R], m32 = __int_as_float(0x7f800000);
-        bool el[R];
+      for (;;) {
+        // Step 1: the most negative reduced cost (Bland: the lowest variable).
+        Im o[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          el[r] = in_m[r] && above(a[r], eps_p);
-          q[r] = el[r] ? __fdiv_rn(d2f_rn(rhs[r]), d2f_rn(a[r])) : __int_as_float(0x7f800000);
-          if (el[r]) m32 = fminf(m32, q[r]);
+          o[r] = in_n[r] && above(neg(obj[r]), eps_d) ? (bland ? Im(0) : image(obj[r])) : kNone;
+          // The random rule: the least key of the variable at this pivot (FP32: of
+          // its upper 31 bits, as the register kernel ranks; RN: of all but the one
+          // value that stands for no candidate).
+          if constexpr (KIND == kRandom)
+            if (o[r] != kNone && !bland) {
+              const unsigned key = rpc_key(P.seed, P.lp_base + lp, iters, int(nkey[r] >> kIdxBits));
+              o[r] = kD ? Im(key) : RN ? Im(min(key, 0xfffffffeu)) : Im(key >> 1);
+            }
         }
-        m32 = ord2f(__reduce_min_sync(kFull, f2ord(m32)));
-        if constexpr (W > 1) {
-          if (lane == 0) fvote[wid] = m32;
-          __syncthreads();
-          m32 = ord2f(__reduce_min_sync(kFull, f2ord(fvote[lane & (W - 1)])));
-        }
-        const float cut = m32 + 1e-5f * fabsf(m32);
-        int cnt = 0;
+        const Cand<T> col = choose(0, o, nkey, obj, obj, cst);
+        if (col.o == kNone) break;
+        if (held == (based ? L.kw : L.kmax)) { full = true; break; }
+        const int e = int(col.key) & kIdxMask, cse = col.last;
+        // Column e: from A (the slot's tableau) or from the pivot that last stood on it,
+        // then the pivots since.
+        T a[R];
+        const int e1 = held < ks ? held : ks;
+        {
+          int s = cse + 1;
+          if (cse < 0 && based) {
+            const T *tab = tableau() + e;
+            const int ld = L.ld;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          el[r] = el[r] && !(q[r] > cut);
-          cnt += el[r];
-        }
-        int all = int(__reduce_add_sync(kFull, unsigned(cnt)));
-        if constexpr (W > 1) {
-          if (lane == 0) votes[wid] = all;
-          __syncthreads();
-          all = 0;
+            for (int r = 0; r < R; ++r) a[r] = tab[ic[r] * ld];
+          } else if (cse < 0) {
 #pragma unroll
-          for (int w = 0; w < W; ++w) all += votes[w];
-        }
-        const bool one = all == 1 && m32 > 4.f * float(eps_p);
+            for (int r = 0; r < R; ++r) a[r] = a_in<T, F64, RN>(A, ic[r] * n + e);
+          } else {
+            const T *h = entry(cse);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          o[r] = kNone;
-          if (__any_sync(kFull, el[r])) {
-            const double t = one ? f2d_exact(q[r]) : rhs[r] / a[r];
-            if (el[r]) o[r] = image(t);
+            for (int r = 0; r < R; ++r) a[r] = neg(h[ic[r]]);
+          }
+#pragma unroll 4
+          for (; s < e1; ++s) {
+            const T *h = hist + s * hs;
+            const T pe = h[pn + e];
+#pragma unroll
+            for (int r = 0; r < R; ++r) a[r] = mul_add(neg(h[ic[r]]), pe, s == rst[r] ? neg_zero<T>() : a[r]);
+          }
+#pragma unroll kSpillUnroll
+          for (; s < held; ++s) {
+            const T *h = spill + (s - ks) * hs;
+            const T pe = h[pn + e];
+#pragma unroll
+            for (int r = 0; r < R; ++r) a[r] = mul_add(neg(h[ic[r]]), pe, s == rst[r] ? neg_zero<T>() : a[r]);
           }
         }
-      } else {
+        // Step 2: the min-ratio test.
+        if constexpr (kD) {
+          // The ratios in FP32 first (relative error below 3e-7; FP64 division is
+          // slow here): only rows within 1e-5 of the smallest get the exact
+          // quotient, and none does when a single row is left whose ratio is
+          // clearly above the degeneracy threshold.
+          float q[R], m32 = __int_as_float(0x7f800000);
+          bool el[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          o[r] = in_m[r] && a[r] > eps_p ? image(T(PACKED ? rhs[r] * recip(a[r]) : RN ? rhs[r] / a[r] : rhs[r] * rcp_approx(float(a[r])))) : kNone;
-      }
-      const Cand<T> row = choose(1, o, bkey, a, rhs, rst);
-      if (row.o == kNone) { status = LPB_UNBOUNDED; break; }
-      if (iters >= max_iter) { status = LPB_ITER_LIMIT; break; }
-      if (held >= L.kmax) { over = true; break; }
-      const int l = int(row.key) & kIdxMask, rsl = row.last;
-      const T rp = recip(row.a), bl = row.b;
-      // Row l: from A or from the pivot that last stood on it, then the pivots since.
-      T p[R];
-      {
-        int s = rsl + 1;
-        if (rsl < 0) {
+          for (int r = 0; r < R; ++r) {
+            el[r] = in_m[r] && above(a[r], eps_p);
+            q[r] = el[r] ? __fdiv_rn(d2f_rn(rhs[r]), d2f_rn(a[r])) : __int_as_float(0x7f800000);
+            if (el[r]) m32 = fminf(m32, q[r]);
+          }
+          m32 = ord2f(__reduce_min_sync(kFull, f2ord(m32)));
+          if constexpr (W > 1) {
+            if (lane == 0) fvote[wid] = m32;
+            __syncthreads();
+            m32 = ord2f(__reduce_min_sync(kFull, f2ord(fvote[lane & (W - 1)])));
+          }
+          const float cut = m32 + 1e-5f * fabsf(m32);
+          int cnt = 0;
 #pragma unroll
-          for (int r = 0; r < R; ++r) p[r] = a_in<T, F64, RN>(A, l * n + jc[r]);
+          for (int r = 0; r < R; ++r) {
+            el[r] = el[r] && !(q[r] > cut);
+            cnt += el[r];
+          }
+          int all = int(__reduce_add_sync(kFull, unsigned(cnt)));
+          if constexpr (W > 1) {
+            if (lane == 0) votes[wid] = all;
+            __syncthreads();
+            all = 0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) all += votes[w];
+          }
+          const bool one = all == 1 && m32 > 4.f * float(eps_p);
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            o[r] = kNone;
+            if (__any_sync(kFull, el[r])) {
+              const double t = one ? f2d_exact(q[r]) : rhs[r] / a[r];
+              if (el[r]) o[r] = image(t);
+            }
+          }
         } else {
-          const T *h = entry(rsl) + pn;
-          const T rs = rps[rsl];
 #pragma unroll
-          for (int r = 0; r < R; ++r) p[r] = h[jc[r]] * rs;
+          for (int r = 0; r < R; ++r)
+            o[r] = in_m[r] && a[r] > eps_p ? image(T(PACKED ? rhs[r] * recip(a[r]) : RN ? rhs[r] / a[r] : rhs[r] * rcp_approx(float(a[r])))) : kNone;
         }
+        const Cand<T> row = choose(1, o, bkey, a, rhs, rst);
+        if (row.o == kNone) { status = LPB_UNBOUNDED; break; }
+        if (iters >= max_iter) { status = LPB_ITER_LIMIT; break; }
+        const int l = int(row.key) & kIdxMask, rsl = row.last;
+        const T rp = recip(row.a), bl = row.b;
+        // Row l likewise.
+        T p[R];
+        {
+          int s = rsl + 1;
+          if (rsl < 0 && based) {
+            const T *tab = tableau() + l * L.ld;
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r] = tab[jc[r]];
+          } else if (rsl < 0) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r] = a_in<T, F64, RN>(A, l * n + jc[r]);
+          } else {
+            const T *h = entry(rsl) + pn;
+            const T rs = rps[rsl];
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r] = h[jc[r]] * rs;
+          }
 #pragma unroll 4
-        for (; s < e1; ++s) {
-          const T *h = hist + s * hs;
-          const T nf = neg(h[l]);
+          for (; s < e1; ++s) {
+            const T *h = hist + s * hs;
+            const T nf = neg(h[l]);
 #pragma unroll
-          for (int r = 0; r < R; ++r) p[r] = mul_add(nf, h[pn + jc[r]], s == cst[r] ? neg_zero<T>() : p[r]);
+            for (int r = 0; r < R; ++r) p[r] = mul_add(nf, h[pn + jc[r]], s == cst[r] ? neg_zero<T>() : p[r]);
+          }
+#pragma unroll kSpillUnroll
+          for (; s < held; ++s) {
+            const T *h = spill + (s - ks) * hs;
+            const T nf = neg(h[l]);
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r] = mul_add(nf, h[pn + jc[r]], s == cst[r] ? neg_zero<T>() : p[r]);
+          }
         }
-#pragma unroll 1
-        for (; s < held; ++s) {
-          const T *h = spill + (s - ks) * hs;
-          const T nf = neg(h[l]);
+        // Step 3 on the right-hand side and the objective row, and the pivot into
+        // the history.
+        T *h = held < ks ? hist + held * hs : spill + (held - ks) * hs;
+        const T fm = col.a * rp;
+        z = mul_add(neg(fm), bl, z);
 #pragma unroll
-          for (int r = 0; r < R; ++r) p[r] = mul_add(nf, h[pn + jc[r]], s == cst[r] ? neg_zero<T>() : p[r]);
+        for (int r = 0; r < R; ++r) {
+          const int i = tid + NT * r;
+          const bool is_l = i == l, is_e = i == e;
+          const T f = is_l ? neg(rp) : a[r] * rp;
+          const T v = is_e ? T(1) : p[r];
+          rhs[r] = mul_add(neg(f), bl, is_l ? neg_zero<T>() : rhs[r]);
+          obj[r] = mul_add(neg(fm), v, is_e ? neg_zero<T>() : obj[r]);
+          if (in_m[r]) h[i] = f;
+          if (in_n[r]) h[pn + i] = v;
+          if (is_l) { bkey[r] = (col.key & ~unsigned(kIdxMask)) | unsigned(l); rst[r] = held; }
+          if (is_e) { nkey[r] = (row.key & ~unsigned(kIdxMask)) | unsigned(e); cst[r] = held; }
+        }
+        if (tid == 0) { rps[held] = rp; ats[held] = unsigned(l << 16 | e); }
+        if constexpr (W == 1) __syncwarp();     // (several warps: the next Step 1's barrier)
+        ++iters;
+        ++held;
+        if (!above(unimage(row.o), eps_p)) {
+          if (++degenerate_run >= m + n) bland = true;
+        } else {
+          degenerate_run = 0;
+          bland = false;
         }
       }
-      // Step 3 on the right-hand side and the objective row, and the pivot into
-      // the history.
-      T *h = held < ks ? hist + held * hs : spill + (held - ks) * hs;
-      const T fm = col.a * rp;
-      z = mul_add(neg(fm), bl, z);
+      sync();
+      // The pivots into the slot's tableau: where no more of them are kept, and for the
+      // refinement of an LP whose earlier ones went there.
+      const bool refines = !kD && !PACKED && P.mode == MODE_FP32_REFINE && status == LPB_OPTIMAL;
+      if (!full && !(refines && based && held > 0)) break;
+      apply_pivots<T, NT, F64, RN>(tableau(), spill, A, m, n, held, based, L.hist, L.at, ks, hs, pn, L.ld);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int i = tid + NT * r;
-        const bool is_l = i == l, is_e = i == e;
-        const T f = is_l ? neg(rp) : a[r] * rp;
-        const T v = is_e ? T(1) : p[r];
-        rhs[r] = mul_add(neg(f), bl, is_l ? neg_zero<T>() : rhs[r]);
-        obj[r] = mul_add(neg(fm), v, is_e ? neg_zero<T>() : obj[r]);
-        if (in_m[r]) h[i] = f;
-        if (in_n[r]) h[pn + i] = v;
-        if (is_l) { bkey[r] = (col.key & ~unsigned(kIdxMask)) | unsigned(l); rst[r] = held; }
-        if (is_e) { nkey[r] = (row.key & ~unsigned(kIdxMask)) | unsigned(e); cst[r] = held; }
-      }
-      if (tid == 0) { rps[held] = rp; ats[held] = unsigned(l << 16 | e); }
-      if constexpr (W == 1) __syncwarp();     // (several warps: the next Step 1's barrier)
-      ++iters;
-      ++held;
-      if (!above(unimage(row.o), eps_p)) {
-        if (++degenerate_run >= m + n) bland = true;
-      } else {
-        degenerate_run = 0;
-        bland = false;
-      }
+      for (int r = 0; r < R; ++r) rst[r] = cst[r] = -1;
+      held = 0;
+      based = true;
+      sync();
+      if (!full) break;
     }
-    sync();
     int bvar[R], nvar[R];          // basic variable of each row, non-basic variable of each column
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -655,12 +918,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     }
     if (status == LPB_ITER_LIMIT) warm_run = -1;
     if (warm && 2 * iters > held) cold_left = kShareChunk - 1;
-    if (over) {
-      warm_run = -1;
-      defer();
-      next();
-      continue;
-    }
+    if (based) warm_run = -1;      // (a warm start runs the pivots from A on)
     const int64_t yoff = P.R.y_off ? P.R.y_off[lp] : boff;    // outputs packed like b, or at y_off
     if (int32_t *bp = P.bbuf ? P.bbuf + (P.bpacked ? yoff : int64_t(lp) * P.B.max_m) : nullptr) {
 #pragma unroll
@@ -728,7 +986,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     }
     double cx = 0.0;
     double *xq = reinterpret_cast<double *>(lz_smem + L.xq);   // [2]: x of the basic structurals, y of the non-basic slacks
-    const int kx = L.kmax;
+    const int kx = L.kx;
     if (!fail) {
       float *dv = reinterpret_cast<float *>(lz_smem + L.dv);     // [2]: residuals, then corrections
       int *off = reinterpret_cast<int *>(lz_smem + L.off);       // [2]: column j_q of A; start of row k_p of A
@@ -760,8 +1018,20 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       const double tp = tol * (1.0 + __longlong_as_double(static_cast<long long>(bm)));
       const double td = tol * (1.0 + __longlong_as_double(static_cast<long long>(cm)));
       constexpr float kDeltaErr = 1.f / 32768.f;
+      if (based) {
+        short *cp = reinterpret_cast<short *>(reinterpret_cast<float *>(hist) + hs), *rq = cp + kx;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (qi[r] >= 0) rq[qi[r]] = short(tid + NT * r);
+          if (pi[r] >= 0) cp[pi[r]] = short(tid + NT * r);
+        }
+        cx = refine_by_tableau<W, F64>(reinterpret_cast<const float *>(tableau()), A, bg, cg, m, n, L.ld, k, kx, L.hist, hs, pn,
+                                       L.xq, L.off, L.kr, L.flag, L.flag + D, L.red + 2 * W * int(sizeof(Cand<T>)) + 16 * W,
+                                       tol, tp, td);
+        fail = cx != cx;
+      }
 #pragma unroll 1
-      for (int round = 0;; ++round) {
+      for (int round = 0; !based; ++round) {
         sync();
         // b - A x by row and A^T y - c by column, in FP64.
         double ra[R], rd[R];
@@ -817,12 +1087,9 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
           v[r] = tr ? v[r] : 0.f;
           w[r] = tc ? w[r] : 0.f;
           // RN: as the tableau kernel does, corrections (three at most) until the
-          // residuals are far below the certificate's bar: 4000 times, because that
-          // kernel asks for 1000 times in the rows of basic slacks too.  (Largest
-          // error in x against FP64, 99% quantile over 10,000 bounded LPs of 100 x
-          // 100: tableau kernel 2.2e-11, here 2.5e-11 with 1000 times.)
+          // residuals are far below the certificate's bar (kStop).
           if constexpr (RN)
-            more |= int(tr && !dge(0.25e-3 * tp, abs_bits(ra[r]))) | int(tc && !dge(0.25e-3 * td, abs_bits(rd[r])));
+            more |= int(tr && !dge(kStop * tp, abs_bits(ra[r]))) | int(tc && !dge(kStop * td, abs_bits(rd[r])));
         }
         bool correct = true;
         if constexpr (RN) correct = any(more) && round < 3;
@@ -997,7 +1264,7 @@ cudaError_t lazy_occ(const LazyConfig (&t)[N], const LazyShape &q, int dtype, in
   const LazyConfig *c = lazy_pick(t, q.max_m > q.max_n ? q.max_m : q.max_n);
   *ctas = 0;
   if (!c) return cudaSuccess;
-  *lay = lazy_layout<T>(q.max_m, q.max_n, c->W, c->R, q.ks, q.kmax);
+  *lay = lazy_layout<T>(q.max_m, q.max_n, c->W, c->R, q.ks, q.kmax, q.kw);
   *threads = 32 * c->W;
   if (lay->bytes > 230000) return cudaSuccess;
   const void *fn = lazy_fn(*c, dtype, q.shared);

@@ -63,3 +63,58 @@ def test_refinement_ends_on_fp64_residuals(solver, m, n, lo):
         td = 1e-12 * (1 + c[k].max()) + (m + 2) * 2.0 ** -53 * float((np.abs(y[k]) @ np.abs(A[k])).max())
         over += rp.max(initial=0) > tp or rd.max(initial=0) > td
     assert over <= resolved
+
+
+GMEM, REG, PACK, WARP = 2, 3, 4, 5
+
+
+def _many_pivots(count, m, n, seed, sparse=False):
+    """LPs with b > 0 whose pivots are of the order of min(m, n): rows of both signs, or one
+    entry in ten."""
+    r = np.random.default_rng(seed)
+    A = r.uniform(0.1, 1, (count, m, n)) * (r.random((count, m, n)) < 0.1) if sparse else r.normal(0.3, 1, (count, m, n))
+    return synth.pack([(A[k], r.uniform(1, 10, m), r.uniform(0, 1, n)) for k in range(count)])
+
+
+# One, two, four and eight warps per LP; LPs that leave the history once and several times;
+# row blocks that are not full; more LPs than CTAs.
+MANY = [(60, 33, 31), (3000, 40, 40), (60, 64, 63), (60, 97, 100), (60, 127, 120), (60, 61, 127), (60, 140, 30),
+        (40, 200, 100), (40, 129, 257), (20, 300, 201)]
+
+
+@pytest.mark.parametrize("count,m,n", MANY)
+@pytest.mark.parametrize("prec,dtype", [("fp64", torch.float64), ("fp64", torch.float32), ("fp32", torch.float64),
+                                        ("fp32", torch.float32), ("fp32_refine", torch.float64),
+                                        ("fp32_refine", torch.float32)])
+@pytest.mark.parametrize("sparse", [False, True])
+def test_many_pivots_as_the_full_update(solver, count, m, n, prec, dtype, sparse):
+    """Pivots applied to the tableau in between: the same operations on every value, so the same
+    pivots and, where results are read straight off, the same bits.  (Refined: an LP whose
+    certificate one rounding of the correction just passes and another does not is solved
+    again, with pivots of its own: one in fifty is left out.)"""
+    sb = _many_pivots(count, m, n, 31 * m + n, sparse)
+    batch = to_device(sb, dtype)
+    full = GMEM if prec == "fp64" or max(m, n) > 127 else WARP if dtype == torch.float64 and m * n <= 10000 else REG
+    got, ref = host(solver.solve(batch, prec=prec)), host(solver.solve(batch, prec=prec, kernel=full))
+    assert np.array_equal(got["status"], ref["status"])
+    assert ref["iters"].max() > 8 + m * n // (m + n) or prec == "fp32_refine"
+    if prec == "fp32_refine":
+        same = (got["iters"] == ref["iters"]) & (got["basis"] == ref["basis"]).reshape(count, m).all(axis=1)
+        assert (~same).sum() <= count // 50
+        ok = ref["status"] == 0
+        assert np.all(np.abs(got["obj"] - ref["obj"])[ok] <= 1e-8 * (1 + np.abs(ref["obj"][ok])))
+    else:
+        for name in ("iters", "basis", "obj", "x", "y"):
+            assert np.array_equal(got[name], ref[name], equal_nan=name == "obj"), name
+    assert solver.sync_error() == 0
+
+
+@pytest.mark.parametrize("m,n", [(31, 31), (20, 29)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_many_pivots_as_several_lps_per_warp(solver, m, n, dtype):
+    sb = _many_pivots(5000, m, n, m + n)
+    batch = to_device(sb, dtype)
+    got, ref = host(solver.solve(batch, prec="fp32")), host(solver.solve(batch, prec="fp32", kernel=PACK))
+    assert ref["iters"].max() > 8 + m * n // (m + n)
+    for name in ("status", "iters", "basis", "obj", "x", "y"):
+        assert np.array_equal(got[name], ref[name], equal_nan=name == "obj"), name
