@@ -43,7 +43,7 @@ namespace {
 using namespace lpb;
 
 // Handle counters (the per-pass work queues live in the workspace).
-enum { CTR_DEFER = 4, CTR_RESOLVE = 5, CTR_BWD = 6, CTR_N = kCounters };
+enum { CTR_OVER = 3, CTR_DEFER = 4, CTR_RESOLVE = 5, CTR_BWD = 6, CTR_N = kCounters };
 
 class DeviceScope {
  public:
@@ -61,7 +61,7 @@ class DeviceScope {
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-enum ListKind { LIST_ALL = 0, LIST_CLASS = 1, LIST_DEFER = 2, LIST_RESOLVE = 3 };
+enum ListKind { LIST_ALL = 0, LIST_CLASS = 1, LIST_DEFER = 2, LIST_RESOLVE = 3, LIST_REST = 4 };
 
 // The launches of the kernel that keeps the pivots.
 // (LAZY_PACK: not under the random rule.)
@@ -88,7 +88,7 @@ struct Pass {
   size_t smem = 0, slot_bytes = 0, tab_smem = 0;
 };
 
-constexpr int kMaxPasses = kMaxClasses + 2;
+constexpr int kMaxPasses = kMaxClasses + 3;
 
 struct Plan {
   Pass pass[kMaxPasses];
@@ -336,7 +336,10 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
     if (p->warp || b->count < 16 * d.sms) return;
     if (kind == LAZY_FP64 ? mx > 8 * mn : kind == LAZY_SMALL ? mx > 64 : q.max_n > 128) return;
   }
-  const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 ? 4 : 3.25) * (!rpc ? 1 : kind == LAZY_FP64 ? 4 : 2);
+  // (Objectives of one polytope beyond it go to the register kernel: no type-1 LP of 50,000 does.)
+  const bool hands_on = shared && kind == LAZY_SMALL;
+  const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 || hands_on ? 4 : 3.25) *
+                      (!rpc ? 1 : kind == LAZY_FP64 ? 4 : 2);
   q.kmax = 2 + int(keep * std::sqrt(double(mn)));
   q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL || kind == LAZY_PACK ? 6 + mn / 10 : 8 + mn / 4;
   const int most = 72 * 1024 / ((q.max_m + q.max_n) * eb);      // a third of an SM's shared memory
@@ -354,7 +357,7 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
   p->lay = lay;
   p->threads = threads;
   p->smem = size_t(lay.bytes);
-  p->slot_bytes = ((size_t(q.kmax - q.ks) * lay.hs + size_t(q.max_m) * lay.ld) * eb + 127) & ~size_t(127);
+  p->slot_bytes = ((size_t(q.kmax - q.ks) * lay.hs + (hands_on ? 0 : size_t(q.max_m) * lay.ld)) * eb + 127) & ~size_t(127);
   p->gmem = true;
   p->grid = occ * d.sms;
   if (p->grid > b->count) p->grid = b->count > 0 ? b->count : 1;
@@ -494,8 +497,14 @@ lpb_err make_plan(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o,
     p.lim_n = b->max_n;
     np = 1;
   }
-  if (!plain)
+  if (!plain) {
+    const Pass first = pl->pass[0];
     for (int i = 0; i < np; ++i) lazy_pass(d, b, o, shared, &pl->pass[i]);
+    if (shared && pl->pass[0].lazy == LAZY_SMALL) {      // what that kernel leaves (one pass, uniform sizes)
+      pl->pass[np] = first;
+      pl->pass[np++].list = LIST_REST;
+    }
+  }
   {                                // LPs that need more artificial columns (Phase I)
     Pass &p = pl->pass[np];
     if ((e = make_pass(d, b, &og, !fp32, b->max_m, mode, plain, &p)) != LPB_OK) return e;
@@ -629,7 +638,12 @@ lpb_err run_solve(const DeviceInfo &d, int32_t *ctr, uint32_t *err, const lpb_ba
     p.lim_m = ps.lim_m;
     p.lim_n = ps.lim_n;
     p.queue = queues + i;
+    p.over_count = ctr + CTR_OVER;
     switch (ps.list) {
+      case LIST_REST:
+        p.in = WorkList{nullptr, p.over_count};
+        p.rest = 1;
+        break;
       case LIST_ALL:
         p.in = WorkList{nullptr, nullptr};
         break;
@@ -759,8 +773,9 @@ namespace {
 // Sizes and offsets of `count` LPs that share A and b (offset 0) and read
 // objective k at k n; y and basis of LP k go to k m of the result.
 __global__ void fill_shared_meta(int32_t *m, int32_t *n, int64_t *a_off, int64_t *b_off, int64_t *c_off,
-                                 int64_t *y_off, int count, int mm, int nn) {
+                                 int64_t *y_off, int32_t *status, int count, int mm, int nn) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
+    status[k] = STATUS_UNSOLVED;
     m[k] = mm;
     n[k] = nn;
     a_off[k] = 0;
@@ -1207,7 +1222,7 @@ lpb_err lpb_solve_shared(lpb_handle *h, int32_t m, int32_t n, int32_t dtype, con
   int64_t *dco = reinterpret_cast<int64_t *>(w + sp.o_co), *dyo = reinterpret_cast<int64_t *>(w + sp.o_yo);
   const int cnt = int(count);
   const int grid = (cnt + 255) / 256 < 4 * d.sms ? (cnt + 255) / 256 : 4 * d.sms;
-  fill_shared_meta<<<grid, 256, 0, s>>>(dm, dn, dao, dbo, dco, dyo, cnt, m, n);
+  fill_shared_meta<<<grid, 256, 0, s>>>(dm, dn, dao, dbo, dco, dyo, r->status, cnt, m, n);
   if (cudaGetLastError() != cudaSuccess) return LPB_ECUDA;
   lpb_batch bt{};
   bt.count = cnt;

@@ -32,6 +32,7 @@ enum : uint32_t {
 
 enum Mode : int { MODE_FP64 = 0, MODE_FP32_REFINE = 1, MODE_FP32 = 2 };
 constexpr int STATUS_PENDING = -1;      // internal: the LP waits for a later pass
+constexpr int STATUS_UNSOLVED = -2;     // internal: an objective of one polytope no kernel has taken
 
 struct BatchDev {
   int count, max_m, max_n, dtype;
@@ -362,6 +363,9 @@ struct TableauParams {
   unsigned long long seed;     // LPB_PIVOT_RPC seed
   long long lp_base;           // batch index of LP 0 of this launch (LPB_PIVOT_RPC keys)
   int shared;                  // every LP shares A and b (lpb_solve_shared): warm starts
+  int32_t *over_count;         // shared, the kernel that keeps the pivots: set to the batch's count
+                               //   when a direction takes more pivots than it keeps
+  int rest;                    // register kernel: only the LPs of status STATUS_UNSOLVED
 };
 
 struct BackwardParams {

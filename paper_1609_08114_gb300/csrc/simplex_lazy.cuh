@@ -38,8 +38,12 @@
 //     kernels.
 //   * Objectives of one polytope (lpb_solve_shared): a CTA takes consecutive ones
 //     and starts each from the basis of the one before, whose history, right-hand
-//     side and variables it keeps: the new objective row is -c run through the
-//     pivots (k n operations).
+//     side and variables it keeps, under either rule and with or without refinement:
+//     the new objective row is -c run through the pivots (k n operations).  Where a
+//     direction takes more than `kmax` pivots, the launch ends, and the register kernel,
+//     whose warm starts cost the same from any basis, solves the objectives left (10,000
+//     directions that turn slowly, 60 x 50 with normal rows, 60 pivots to the first
+//     optimum: 0.71 ms on that kernel, 0.82 here, 1.2 through a tableau in the slot).
 //
 // What bounds it, at 50,000 x 100 with FP64 input (4.19 ms on the kernel that updates
 // the whole tableau -> 2.06 ms, 0.30 of the copy bandwidth over the 83.6 KB that an LP
@@ -73,7 +77,7 @@ constexpr int kApplyRows = 8;
 // 100 x 100: tableau kernel 2.2e-11; here 2.5e-11 with its 1e-3, 1.2e-11 with this.)
 constexpr double kStop = 0.25e-3;
 constexpr int kApplyCols = 2;
-enum : int { kCommon = 0, kShared = 1, kRandom = 2, kPacked = 3 };
+enum : int { kCommon = 0, kShared = 1, kRandom = 2, kPacked = 4 };
 
 __device__ __forceinline__ float neg(float v) { return -v; }
 __device__ __forceinline__ double neg(double v) { return neg_bits(v); }
@@ -429,7 +433,7 @@ __device__ __noinline__ double refine_by_tableau(const float *tab, const void *A
 // input's type; RN: the tableau kernel's arithmetic (input rounded, exact
 // ratios) instead of the register kernel's (input truncated, approximate ones).
 // KIND: kShared (objectives of one polytope, with warm starts), kRandom (the
-// random entering rule) and kPacked (with RN: the arithmetic of the
+// random entering rule), both, and kPacked (with RN: the arithmetic of the
 // several-LPs-per-warp kernel, ratios by the rounded reciprocal, and no
 // refinement) are their own instantiations, so that the common one carries none of them.
 template <typename T, int W, int R, int MINB, bool F64, bool RN, int KIND>
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   using In = std::conditional_t<F64, double, float>;
   using Im = Img<T>;
   constexpr int NT = 32 * W, D = NT * R;
-  constexpr bool kD = sizeof(T) == 8, SHARED = KIND == kShared, PACKED = KIND == kPacked;
+  constexpr bool kD = sizeof(T) == 8, SHARED = (KIND & kShared) != 0, PACKED = KIND == kPacked;
   constexpr int kSpillUnroll = kD ? 1 : RN ? 4 : 2;    // history entries in flight from the workspace
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
   constexpr Im kNone = Im(~Im(0));
@@ -524,21 +528,26 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   int warm_run = 0;                // objectives since a cold start; -1: the history is no basis of this polytope
   bool scanned = false;            // the shared A is known to be finite
   int cold_left = 0;               // objectives to start cold, since a warm start took many pivots
+  int cold_iters = 0;              // pivots of the last cold start
+  int nitem = 0;
+  bool again = false;              // the same objective once more, cold
 #pragma unroll 1
   while (item < nitems) {
-    int nitem = 0;
-    if (tid == 0) nitem = claim(item);
+    if (tid == 0 && !(SHARED && again)) {
+      nitem = claim(item);
+      // Another CTA has met a direction of many pivots: none after this one here either.
+      if (SHARED && *static_cast<volatile int32_t *>(P.over_count) != 0) nitem = nitems;
+    }
+    again = false;
     // ---- admission: sizes, b >= 0, finite data in the tableau's range ----
     const In *A = static_cast<const In *>(P.B.A) + aoff;
     const In *bg = static_cast<const In *>(P.B.b) + boff, *cg = static_cast<const In *>(P.B.c) + coff;
     const bool fits = fits_lp(m, n);
     int bad = !fits;
-    // A warm start keeps the basis of the objective before: while few pivots
-    // lead to it (chains run over all of them), for a bounded number of
-    // objectives (FP32 round-off grows with the pivots), and not where the
+    // A warm start keeps the basis of the objective before: for a bounded number
+    // of objectives (FP32 round-off grows with the pivots), and not where the
     // directions have little to do with one another.
-    const bool warm = SHARED && P.mode == MODE_FP32_REFINE && warm_run >= 0 && warm_run < kWarmMax && held > 0 &&
-                      held <= ks && cold_left == 0;
+    const bool warm = SHARED && warm_run >= 0 && warm_run < kWarmMax && held > 0 && cold_left == 0;
     if (SHARED && cold_left > 0) --cold_left;
     unsigned long long cm = 0ull;
     int ic[R], jc[R];              // own rows and columns; past the end the last one (read, never used)
@@ -720,14 +729,38 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     const int max_iter = P.max_iter > 0 ? P.max_iter : 50 * (m + n);
     int iters = 0, status = LPB_OPTIMAL, degenerate_run = 0;
     T z = T(0);
-    if (warm) {                    // the new objective row on the basis kept: -c through its pivots
-      sync();
-      if constexpr (SHARED) through_pivots(nullptr, obj);
+    if constexpr (SHARED) {
+      if (warm) {                  // the new objective row on the basis kept: -c through its pivots
+        sync();
+        through_pivots(nullptr, obj);
+        if (P.mode == MODE_FP32) { // and z = c_B x_B (refinement forms its own)
+          float part = 0.f;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int v = int(bkey[r] >> kIdxBits);
+            int none = 0;
+            if (in_m[r] && v < n) {
+              if constexpr (F64) part = fmaf(d2f_tile(__ldg(cg + v), none), rhs[r], part);
+              else part = fmaf(__ldg(cg + v), rhs[r], part);
+            }
+          }
+#pragma unroll
+          for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
+          if constexpr (W > 1) {
+            if (lane == 0) fvote[wid] = part;
+            __syncthreads();
+            part = 0.f;
+#pragma unroll
+            for (int w = 0; w < W; ++w) part += fvote[w];
+          }
+          z = part;
+        }
+      }
     }
-    bool bland = false;
+    bool bland = false, full = false;
 #pragma unroll 1
     for (;;) {
-      bool full = false;
+      full = false;
 #pragma unroll 1
       for (;;) {
         // Step 1: the most negative reduced cost (Bland: the lowest variable).
@@ -738,7 +771,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
           // The random rule: the least key of the variable at this pivot (FP32: of
           // its upper 31 bits, as the register kernel ranks; RN: of all but the one
           // value that stands for no candidate).
-          if constexpr (KIND == kRandom)
+          if constexpr ((KIND & kRandom) != 0)
             if (o[r] != kNone && !bland) {
               const unsigned key = rpc_key(P.seed, P.lp_base + lp, iters, int(nkey[r] >> kIdxBits));
               o[r] = kD ? Im(key) : RN ? Im(min(key, 0xfffffffeu)) : Im(key >> 1);
@@ -901,7 +934,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       // The pivots into the slot's tableau: where no more of them are kept, and for the
       // refinement of an LP whose earlier ones went there.
       const bool refines = !kD && !PACKED && P.mode == MODE_FP32_REFINE && status == LPB_OPTIMAL;
-      if (!full && !(refines && based && held > 0)) break;
+      if (SHARED || (!full && !(refines && based && held > 0))) break;
       apply_pivots<T, NT, F64, RN>(tableau(), spill, A, m, n, held, based, L.hist, L.at, ks, hs, pn, L.ld);
 #pragma unroll
       for (int r = 0; r < R; ++r) rst[r] = cst[r] = -1;
@@ -910,6 +943,15 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       sync();
       if (!full) break;
     }
+    if (SHARED && full) {
+      if (warm) {                  // the history is full after some warm starts: cold
+        again = true;
+        warm_run = -1;
+        continue;
+      }
+      if (tid == 0) *P.over_count = P.B.count;      // many pivots: the register kernel's launch
+      break;                                        // solves what has no status yet
+    }
     int bvar[R], nvar[R];          // basic variable of each row, non-basic variable of each column
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -917,8 +959,8 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       nvar[r] = int(nkey[r] >> kIdxBits);
     }
     if (status == LPB_ITER_LIMIT) warm_run = -1;
-    if (warm && 2 * iters > held) cold_left = kShareChunk - 1;
-    if (based) warm_run = -1;      // (a warm start runs the pivots from A on)
+    if (!warm) cold_iters = iters;
+    if (warm && 2 * iters > cold_iters) cold_left = kShareChunk - 1;
     const int64_t yoff = P.R.y_off ? P.R.y_off[lp] : boff;    // outputs packed like b, or at y_off
     if (int32_t *bp = P.bbuf ? P.bbuf + (P.bpacked ? yoff : int64_t(lp) * P.B.max_m) : nullptr) {
 #pragma unroll
@@ -1240,7 +1282,7 @@ struct LazyConfig {
 
 template <typename T, int W, int R, int MINB, bool RN, int KIND = kCommon>
 constexpr LazyConfig lazy_config() {
-  constexpr int kS = sizeof(T) == 4 && !RN && KIND == kCommon ? int(kShared) : KIND;
+  constexpr int kS = sizeof(T) == 4 && !RN ? KIND | kShared : KIND;
   return LazyConfig{W, R, reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, KIND>),
                     reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, false, RN, KIND>),
                     reinterpret_cast<const void *>(&lazy_kernel<T, W, R, MINB, true, RN, kS>),

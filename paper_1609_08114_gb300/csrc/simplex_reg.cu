@@ -346,9 +346,17 @@ __global__ void __launch_bounds__(W * 32, reg_min_blocks<R, C, W>()) reg_kernel(
     if (item >= nitems) break;
     const bool pre = sh.pre != 0;          // reset by thread 0 after the next barrier
     const bool warm = sh.warm_ok != 0;     // keep the basis; load and price only the new objective
+    const int lp = D.lp;
+    if (P.rest && P.R.status[lp] != STATUS_UNSOLVED) {    // solved by the launch before
+      if (tid == claimer) {
+        next = claim(item);
+        sh.cstage = 0;
+      }
+      __syncthreads();
+      continue;
+    }
     warm_run = warm ? warm_run + 1 : 0;
     valid_tab = 0;
-    const int lp = D.lp;
     const int m = D.m, n = D.n;
     const int64_t aoff = D.aoff, boff = D.boff, coff = D.coff;
     // ---- admission: sizes that fit the template, b >= 0, finite b and c ----

@@ -118,3 +118,28 @@ def test_many_pivots_as_several_lps_per_warp(solver, m, n, dtype):
     assert ref["iters"].max() > 8 + m * n // (m + n)
     for name in ("status", "iters", "basis", "obj", "x", "y"):
         assert np.array_equal(got[name], ref[name], equal_nan=name == "obj"), name
+
+
+@pytest.mark.parametrize("prec,rtol", [("fp32", 1e-4), ("fp32_refine", 1e-8)])
+@pytest.mark.parametrize("rule", ["lpc", "rpc"])
+@pytest.mark.parametrize("m,n,normal", [(40, 33, False), (64, 64, False), (33, 31, True), (60, 50, True), (100, 90, True)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_warm_starts_in_every_mode(solver, prec, rtol, rule, m, n, normal, dtype):
+    """Directions that turn slowly, on polytopes whose optimal bases take few pivots and many
+    (rows of both signs): each objective starts from the one before under either rule, with
+    and without refinement, in batches that fill the GPU (the random rule's route).  Plain FP32:
+    some 64 warm pivots and 64 cold ones at 2^-24 times values up to 100, against FP64."""
+    r = np.random.default_rng(m + n)
+    A = r.normal(0.3, 1, (m, n)) if normal else r.uniform(0.1, 1, (m, n))
+    b, count = r.uniform(1, 10, m), 2500
+    C = r.uniform(0.1, 1, n)[None] + 1e-5 * np.arange(count)[:, None] * r.normal(size=n)[None]
+    args = [torch.tensor(v, device="cuda", dtype=dtype) for v in (A, b, C)]
+    got = host(solver.solve_shared(*args, prec=prec, pivot_rule=rule, seed=3))
+    ref = host(solver.solve_shared(*[a.double() for a in args], prec="fp64", pivot_rule=rule, seed=3))
+    assert np.array_equal(got["status"], ref["status"]) and (ref["status"] == 0).all()
+    assert np.all(np.abs(got["obj"] - ref["obj"]) <= rtol * (1 + np.abs(ref["obj"])))
+    x, y = got["x"].reshape(count, n), got["y"].reshape(count, m)
+    Ad, bd, Cd = (a.double().cpu().numpy() for a in args)
+    assert (x @ Ad.T - bd).max() <= rtol * 100 and (Cd - y @ Ad).max() <= rtol * 100 and min(x.min(), y.min()) >= -rtol * 100
+    assert got["iters"].mean() < 0.3 * ref["iters"].mean()
+    assert solver.sync_error() == 0
