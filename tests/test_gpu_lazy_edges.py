@@ -143,3 +143,56 @@ def test_warm_starts_in_every_mode(solver, prec, rtol, rule, m, n, normal, dtype
     assert (x @ Ad.T - bd).max() <= rtol * 100 and (Cd - y @ Ad).max() <= rtol * 100 and min(x.min(), y.min()) >= -rtol * 100
     assert got["iters"].mean() < 0.3 * ref["iters"].mean()
     assert solver.sync_error() == 0
+
+
+# The configurations of 385 to 1,024 rows or columns (eight warps; two and four rows or columns
+# per thread), where most of the history lies in the workspace.
+@pytest.mark.parametrize("count,m,n", [(12, 385, 40), (12, 512, 30), (12, 513, 40), (12, 40, 1000), (8, 1024, 20),
+                                       (6, 530, 600)])
+@pytest.mark.parametrize("prec,dtype", [("fp64", torch.float64), ("fp32", torch.float32), ("fp32_refine", torch.float64)])
+@pytest.mark.parametrize("many", [False, True])
+def test_largest_configurations(solver, count, m, n, prec, dtype, many):
+    """LPs of few pivots and (one entry in ten) of many, as above."""
+    sb = _many_pivots(count, m, n, m + n, sparse=True) if many else synth.type1(count, m, n, seed=m + n)
+    batch = to_device(sb, dtype)
+    got, ref = host(solver.solve(batch, prec=prec)), host(solver.solve(batch, prec=prec, kernel=GMEM))
+    assert np.array_equal(got["status"], ref["status"])
+    if prec == "fp32_refine":
+        assert (got["iters"] != ref["iters"]).sum() <= 1       # (an LP solved again, as above)
+        ok = ref["status"] == 0
+        assert np.all(np.abs(got["obj"][ok] - ref["obj"][ok]) <= 1e-8 * (1 + np.abs(ref["obj"][ok])))
+    else:
+        for name in ("iters", "basis", "obj", "x", "y"):
+            assert np.array_equal(got[name], ref[name], equal_nan=name == "obj"), name
+    assert solver.sync_error() == 0
+
+
+@pytest.mark.parametrize("m,n,prec", [(520, 66, "fp64"), (400, 51, "fp64"), (520, 20, "fp32"), (400, 20, "fp32_refine")])
+def test_largest_configurations_under_the_random_rule(solver, m, n, prec):
+    """In a batch that fills the GPU: a CTA runs many LPs, one after another."""
+    sb = synth.type1(2500, m, n, seed=m)
+    batch = to_device(sb)
+    got = host(solver.solve(batch, prec=prec, pivot_rule="rpc", seed=5))
+    ref = host(solver.solve(batch, prec=prec, pivot_rule="rpc", seed=5, kernel=GMEM))
+    assert np.array_equal(got["status"], ref["status"])
+    if prec == "fp32_refine":
+        assert (got["iters"] != ref["iters"]).sum() <= 50
+    else:
+        for name in ("iters", "basis", "obj", "x", "y"):
+            assert np.array_equal(got[name], ref[name]), name
+    assert np.all(np.abs(got["obj"] - ref["obj"]) <= 1e-8 * (1 + np.abs(ref["obj"])))
+    assert solver.sync_error() == 0
+
+
+@pytest.mark.parametrize("count,m,n,prec", [(6000, 33, 31, "fp64"), (4000, 64, 40, "fp64"), (2000, 130, 24, "fp64"),
+                                            (6000, 60, 64, "fp32"), (4000, 100, 70, "fp32"), (2500, 140, 30, "fp32")])
+def test_nothing_is_left_from_one_lp_to_the_next(solver, count, m, n, prec):
+    """Several LPs per CTA, every other one of many pivots."""
+    few, many = synth.type1(count, m, n, seed=m), _many_pivots(count, m, n, n)
+    sb = synth.pack([(many if k % 2 else few).lp(k) for k in range(count)])
+    batch = to_device(sb)
+    full = GMEM if prec == "fp64" or max(m, n) > 127 else WARP
+    got, ref = host(solver.solve(batch, prec=prec)), host(solver.solve(batch, prec=prec, kernel=full))
+    for name in ("status", "iters", "basis", "obj", "x", "y"):
+        assert np.array_equal(got[name], ref[name], equal_nan=name == "obj"), name
+    assert solver.sync_error() == 0
