@@ -196,3 +196,54 @@ def test_nothing_is_left_from_one_lp_to_the_next(solver, count, m, n, prec):
     for name in ("status", "iters", "basis", "obj", "x", "y"):
         assert np.array_equal(got[name], ref[name], equal_nan=name == "obj"), name
     assert solver.sync_error() == 0
+
+
+@pytest.mark.parametrize("call", ["solve", "shared", "bounded", "host"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32_refine"])
+def test_less_workspace_in_every_call(call, prec):
+    """256 bytes less than asked for: the kernels that update the whole tableau, with the same
+    statuses and pivots (warm starts of one polytope's objectives: the same optima).  Far
+    less: refused."""
+    from paper_1609_08114_gb300 import LPBatch, Solver, _lib
+    from paper_1609_08114_gb300._lib import LPBError
+
+    class Short(Solver):
+        cut, asked = 0, []
+
+        def workspace(self, nbytes):
+            self.asked.append(nbytes)
+            return torch.empty(max(256, nbytes - self.cut), dtype=torch.uint8, device="cuda")
+
+    s, count, m, n = Short(0), 2500, 90, 80
+    sb = synth.type1(count, m, n, seed=8)
+    batch = to_device(sb)
+    pinned = LPBatch(*(t.cpu().pin_memory() for t in (batch.m, batch.n, batch.a_off, batch.b_off, batch.c_off, batch.A,
+                                                      batch.b, batch.c)), batch.max_m, batch.max_n, batch.min_m, batch.min_n)
+    run = {"solve": lambda: s.solve(batch, prec=prec), "host": lambda: s.solve_host(pinned, prec=prec, chunk=1000),
+           "shared": lambda: s.solve_shared(batch.A[:m * n].view(m, n), batch.b[:m], batch.c.view(count, n), prec=prec),
+           "bounded": lambda: s.solve_bounded(batch, torch.zeros_like(batch.c), torch.full_like(batch.c, 0.2), prec=prec)}[call]
+
+    def result():
+        r = run()
+        torch.cuda.synchronize()
+        return {k: getattr(r, k).cpu().numpy().copy() for k in ("status", "iters", "obj")}
+
+    want, kernels = result(), s.stats()["kernels"]
+    s.cut = 256
+    if call == "bounded" and prec == "fp32_refine":    # its Phase-I slots are the larger ones: nothing to do without
+        with pytest.raises(LPBError) as e:
+            result()
+        assert e.value.code == _lib.ENOMEM
+        return
+    got = result()
+    assert (want["status"] == 0).all() and np.array_equal(got["status"], want["status"])
+    if call == "shared" and prec == "fp32_refine":
+        assert s.stats()["kernels"] == kernels - 1     # the launch for what the first one leaves
+    else:
+        assert np.array_equal(got["iters"], want["iters"])
+    assert np.all(np.abs(got["obj"] - want["obj"]) <= 1e-8 * (1 + np.abs(want["obj"])))
+    s.cut = 1 << 40
+    with pytest.raises(LPBError) as e:
+        result()
+    assert e.value.code == _lib.ENOMEM
+    assert s.sync_error() == 0
