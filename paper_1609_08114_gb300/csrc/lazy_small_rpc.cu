@@ -1,14 +1,14 @@
-// lazy_small_rpc.cu -- the pivots kept, FP32, the register kernel's arithmetic (m, n <= 127), random entering rule.
+// lazy_small_rpc.cu -- the pivots kept, FP32, the register kernel's arithmetic (m, n <= 64), random entering rule.
 #include "simplex_lazy.cuh"
 
 namespace lpb {
 
 namespace {
-// Warps per LP, rows and columns per thread, CTAs per SM at least.
+// Warps per LP, rows and columns per thread, CTAs per SM at least.  (Above 64 rows or
+// columns the planner leaves this rule to the other kernels.)
 const LazyConfig kTable[] = {
     lazy_config<float, 1, 1, 16, false, kRandom>(),
     lazy_config<float, 1, 2, 16, false, kRandom>(),
-    lazy_config<float, 2, 2, 8, false, kRandom>(),
 };
 }  // namespace
 

@@ -63,15 +63,15 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 enum ListKind { LIST_ALL = 0, LIST_CLASS = 1, LIST_DEFER = 2, LIST_RESOLVE = 3, LIST_REST = 4 };
 
-// The launches of the kernel that keeps the pivots.
-// (LAZY_PACK: not under the random rule.)
+// The launches of the kernel that keeps the pivots (LAZY_PACK: not under the
+// random rule).
 enum LazyKind { LAZY_SMALL = 0, LAZY_LARGE = 1, LAZY_FP64 = 2, LAZY_PACK = 3, LAZY_NONE = -1 };
 constexpr decltype(&lazy_occupancy_small) kLazyOccupancy[2][4] = {
     {lazy_occupancy_small, lazy_occupancy_large, lazy_occupancy_fp64, lazy_occupancy_pack},
-    {lazy_occupancy_small_rpc, lazy_occupancy_large_rpc, lazy_occupancy_fp64_rpc, lazy_occupancy_pack}};
+    {lazy_occupancy_small_rpc, lazy_occupancy_large_rpc, lazy_occupancy_fp64_rpc, nullptr}};
 constexpr decltype(&launch_lazy_small) kLaunchLazy[2][4] = {
     {launch_lazy_small, launch_lazy_large, launch_lazy_fp64, launch_lazy_pack},
-    {launch_lazy_small_rpc, launch_lazy_large_rpc, launch_lazy_fp64_rpc, launch_lazy_pack}};
+    {launch_lazy_small_rpc, launch_lazy_large_rpc, launch_lazy_fp64_rpc, nullptr}};
 
 struct Pass {
   bool fp64 = false, gmem = false;
@@ -280,18 +280,24 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // (simplex_lazy.cuh), with the arithmetic of the kernel that had the pass, so
 // the pivots are the same.  Every size up to 1024 under the largest-coefficient
 // rule, unless a kernel shape is asked for or several LPs share a warp: measured
-// faster at every size tried (type-1 LPs, ms per solve before and after):
-//   30,000 x 48 x 37, FP32 input   1.43 -> 0.28    50,000 x 64    1.46 -> 0.68
-//   50,000 x 100                   4.19 -> 2.11    2,000 x 300    6.0 -> 1.8-2.1
-//   20,000 x 100, FP64 tableau    12.42 -> 1.38
+// faster at every size tried at the pivots of type-1 LPs (ms per solve before and after):
+//   30,000 x 48 x 37, FP32 input   1.43 -> 0.29    50,000 x 64    1.46 -> 0.73
+//   50,000 x 100                   4.19 -> 2.03    2,000 x 300    6.0 -> 1.4-1.6
+//   20,000 x 100, FP64 tableau    12.42 -> 1.37
+// and, with many pivots (normal rows, 70 to 310), everywhere but in plain FP32
+// at 65 to 127 rows or columns with FP64 input, where the warp kernel's tableau in
+// shared memory stays ahead (20,000 LPs or as said, ms before and after):
+//   100, FP64 tableau       101 -> 58     4,000 x 200 x 100       14.9 -> 7.0
+//   64, FP64 tableau       30.7 -> 13.6   64 x 64, FP32 input      6.4 -> 3.2
+//   100, plain FP32         8.6 -> 9.9    64 x 64, plain FP32      2.4 -> 2.3
 // Of the several-LPs-per-warp kernel's passes those of plain FP32 with one or two
 // LPs per warp come here (100,000 LPs: 28 x 28 0.82 -> 0.25, 16 x 31 with FP32
 // input 0.87 -> 0.20, 15 x 15 0.22 -> 0.17, 12 x 12 0.19 -> 0.16, 8 x 8 0.15 ->
 // 0.13; 10,000 x 28 0.099 -> 0.052), from as many LPs on as take longer than the
 // host takes to plan and launch (10,000 x 12 0.048 and 0.050, 1,000 x 30 x 20
-// 0.047 and 0.049).  With four (m, n <= 7) that kernel's lanes are full.  Its refinement corrects by products with the final
-// tableau, which this kernel mostly does not have: another rounding of the results,
-// so refined passes stay.
+// 0.047 and 0.049).  With four (m, n <= 7) that kernel's lanes are full.  Its
+// refinement corrects by products with the final tableau, which this kernel mostly
+// does not have: another rounding of the results, so refined passes stay.
 // The random rule takes over three times the pivots (45.6 against 13.3 at
 // 100 x 100), so its chains are longer and a full update is the better one in
 // places: it comes here only with enough LPs to fill the GPU (300 x 100 FP64 0.98

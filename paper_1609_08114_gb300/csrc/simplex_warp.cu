@@ -50,7 +50,7 @@ namespace {
 constexpr int kWarpMaxWarps = 8;      // LPs (warps) per CTA at most
 constexpr int kWarpMaxDim = 127;      // largest m and n: four rows (columns) per lane
 constexpr int kNoKey = 1 << 30;       // a key larger than any real key
-constexpr int kRefK = 24;             // basic structurals the on-chip refinement takes at most
+constexpr int kRefK = kWarpRefK;      // basic structurals the on-chip refinement takes at most
 
 // One warp's region of shared memory.
 struct WarpLayout {
