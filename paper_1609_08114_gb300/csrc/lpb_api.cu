@@ -289,7 +289,7 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // shared memory stays ahead (20,000 LPs or as said, ms before and after):
 //   100, FP64 tableau       101 -> 58     4,000 x 200 x 100       14.9 -> 7.0
 //   64, FP64 tableau       30.7 -> 13.6   64 x 64, FP32 input      6.4 -> 3.2
-//   100, plain FP32         8.6 -> 9.9    64 x 64, plain FP32      2.4 -> 2.3
+//   100, plain FP32         8.6 -> 9.4    64 x 64, plain FP32      2.4 -> 2.3
 // Of the several-LPs-per-warp kernel's passes those of plain FP32 with one or two
 // LPs per warp come here (100,000 LPs: 28 x 28 0.82 -> 0.25, 16 x 31 with FP32
 // input 0.87 -> 0.20, 15 x 15 0.22 -> 0.17, 12 x 12 0.19 -> 0.16, 8 x 8 0.15 ->
@@ -317,13 +317,18 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // LPs take at most (39 of 50,000 at 100 x 100, 30 at 64 x 64, 22 at 48 x 37, 69 at
 // 300 x 300: about 4 sqrt(min(m, n)); under the random rule two to four times
 // that), which an application would cost more than the chains.  LPs of many pivots
-// would have it earlier, as the entries beyond the shared ones come from L2 (20,000 x
-// 100 x 100, normal rows, 126 pivots, plain FP32: 9.5 ms with 27, 9.9 with 34, 10.2
-// with 37, where 50,000 type-1 LPs take 2.25, 2.13, 2.14).  FP64: 58 ms with 42, 63
-// with 58 (type-1 1.6 ms with 32, 1.37 with 42).  Four and eight warps per LP: 4,000 x
-// 200 x 100 with one entry in ten, 102 pivots, 4.2 ms with 42, 5.0 with 72, 5.4 with
-// 100; 10,000 LPs with a bound on every variable, 64 pivots, 9.2, 8.2, 7.9.  The
-// kernels that update the whole tableau: 8.6 (plain FP32), 101 (FP64), 10.0 and 17.7 ms.
+// would have it earlier, as the entries beyond the shared ones come from L2.  ms with
+// so many kept (normal: normal rows, 126 pivots at 100 x 100; tenth: one entry in ten,
+// 102 pivots at 200 x 100; last: with a full update per pivot):
+//   50,000 x 100 type 1, refined        27: 2.25   34: 2.13   37: 2.14    4.19
+//   40,000 x 100 type 1, plain FP32     22: 1.42   26: 1.33   34: 1.35    2.58
+//   20,000 x 100 normal, plain FP32     22: 9.3    26: 9.4    34: 9.9     8.6
+//   40,000 x 31 type 1, plain FP32      15: 0.220             20: 0.217   0.468
+//   20,000 x 31 normal, plain FP32      15: 0.503             20: 0.533   0.503
+//   20,000 x 100 type 1, FP64           32: 1.6    42: 1.37   58: 1.37   12.4
+//   20,000 x 100 normal, FP64                      42: 58     58: 63    101
+//   4,000 x 200 x 100 tenth, refined    42: 4.2    72: 5.0   100: 5.4    10.0
+//   10,000 x 100 bounded, 64 pivots     42: 9.2    72: 8.2   100: 7.9    17.7
 void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int shared, Pass *p) {
   if ((o->kernel != LPB_KERNEL_AUTO && shared != 2) || o->threads != 0 || o->reg_warps != 0) return;
   if (o->pivot_rule == LPB_PIVOT_STEEPEST) return;
@@ -344,7 +349,8 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
   }
   // (Objectives of one polytope beyond it go to the register kernel: no type-1 LP of 50,000 does.)
   const bool hands_on = shared && kind == LAZY_SMALL;
-  const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 || hands_on ? 4 : 3.25) *
+  const bool plain = p->mode == MODE_FP32 && (kind == LAZY_PACK || (q.max_m > q.max_n ? q.max_m : q.max_n) > 64);
+  const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 || hands_on ? 4 : plain ? 2.5 : 3.25) *
                       (!rpc ? 1 : kind == LAZY_FP64 ? 4 : 2);
   q.kmax = 2 + int(keep * std::sqrt(double(mn)));
   q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL || kind == LAZY_PACK ? 6 + mn / 10 : 8 + mn / 4;

@@ -28,7 +28,7 @@
 //     slot's entries.  The order of operations on an entry is the same, so are the
 //     values.  (20,000 x 100 x 100 with normal rows, 126 pivots: FP64 134 ms when such
 //     LPs started again in the tableau kernel, 58 now, 101 with a full update per pivot;
-//     plain FP32 28.9, 9.9 and 8.6.)
+//     plain FP32 28.9, 9.4 and 8.6.)
 //   * A is read where it lies: one pass over it checks that it is finite (and
 //     leaves it in L2), then a pivot reads the one row and column it needs.
 //   * Refinement and certificate (FP32 + refinement): FP64 residuals from A; the
