@@ -130,6 +130,10 @@ int auto_threads(int eb, int rows, int cols, size_t smem) {
 // with, 6,000 LPs: 24 x 24 1.08 and 1.23, 30 x 40 1.61 and 1.54, 60 x 20 2.81 and
 // 2.30, 60 x 60 6.2 and 3.7, 80 x 80 16.2 and 9.8; 4,000 x 200 x 200 193 and 71).
 // FP64 does not gain: its update is bound by the FP64 pipe, not by the sweeps.
+// The 64 KB are room for two CTAs per SM with tableau rows beside the arrays, not a
+// crossover: past them (from about 296 x 296) deferring would still be the faster one
+// (two-phase LPs in plain FP32, ms with this limit and with 100 KB: 1,200 x 280 x 280 113 and
+// 113, 1,200 x 300 x 300 283 and 137, 600 x 400 x 400 786 and 213).
 bool tableau_defers(const lpb_batch *b, const lpb_options *o, bool fp64, int kcap) {
   if (fp64 || o->kernel != LPB_KERNEL_AUTO || o->threads != 0 || o->pivot_rule != LPB_PIVOT_LPC) return false;
   if (tableau_fixed_bytes(4, b->max_m, b->max_n, kcap, false, true) -

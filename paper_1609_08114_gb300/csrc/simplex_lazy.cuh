@@ -46,15 +46,16 @@
 //     optimum: 0.71 ms on that kernel, 0.82 here, 1.2 through a tableau in the slot).
 //
 // What bounds it, at 50,000 x 100 with FP64 input (4.19 ms on the kernel that updates
-// the whole tableau -> 2.06 ms, 0.30 of the copy bandwidth over the 83.6 KB that an LP
-// must move): the waits of each pivot on A's column and row, with 16 warps per SM to
-// hide them (scheduler slots 41% used, `long_scoreboard` 3.6 of 9 cycles per
-// instruction); 113 KB of DRAM traffic per LP, because L2 has let go of a part of A by
-// the time a pivot gathers from it.  That is also why an LP has two warps and eight LPs
-// an SM, and nothing is fetched ahead: one warp per LP and nine LPs, or fetching the next
-// LP, read A up to three times from DRAM (3.4 ms).  A one-time FP32 copy of A in shared
-// memory takes away the LPs in flight (2.45 ms at best).  FP64 tableau, 20,000 x 100
-// (12.4 -> 1.37 ms): the FP64 pipe, 69% busy.
+// the whole tableau -> 2.03 ms, 0.30 of the copy bandwidth over the 83.6 KB that an LP
+// must move): the serial steps of a pivot -- two arg-mins with a barrier each, the column
+// and the row from where A lies, their chains -- some 5,000 cycles of which 16 warps per
+// SM hide the most part (scheduler slots 41% used).  Not A's traffic alone: 50,000 directions
+// of one polytope, whose A stays in L2 and is read through once, take 1.85 ms.  But L2 lets
+// go of a part of A by the time a pivot gathers from it (113 KB of DRAM traffic per LP),
+// which is why an LP has two warps and eight LPs an SM, and nothing is fetched ahead: one
+// warp per LP and nine LPs, or fetching the next LP, read A up to three times from DRAM
+// (3.4 ms).  A one-time FP32 copy of A in shared memory takes away the LPs in flight (2.45
+// ms at best).  FP64 tableau, 20,000 x 100 (12.4 -> 1.37 ms): the FP64 pipe, 69% busy.
 #pragma once
 #include <type_traits>
 
@@ -68,15 +69,15 @@ namespace {
 // between two cold ones.
 constexpr int kShareChunk = 16;
 constexpr int kWarmMax = 32;
-// Rows of a column that a thread takes at a time when pivots are applied (the
-// history's pivot rows start at a multiple of it).
+// Rows and (FP32) columns that a thread takes at a time when pivots are applied (the
+// history's pivot rows start at a multiple of the rows).
 constexpr int kApplyRows = 8;
+constexpr int kApplyCols = 2;
 // Residuals, in parts of the certificate's bar, at which refinement stops (the tableau
 // kernel's arithmetic): a quarter of that kernel's, which asks for it in the rows of
 // basic slacks too.  (Error in x against FP64, 99% quantile over 10,000 bounded LPs of
 // 100 x 100: tableau kernel 2.2e-11; here 2.5e-11 with its 1e-3, 1.2e-11 with this.)
 constexpr double kStop = 0.25e-3;
-constexpr int kApplyCols = 2;
 enum : int { kCommon = 0, kShared = 1, kRandom = 2, kPacked = 4 };
 
 __device__ __forceinline__ float neg(float v) { return -v; }
