@@ -327,7 +327,7 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 //   50,000 x 100 type 1, refined        27: 2.25   34: 2.13   37: 2.14    4.19
 //   40,000 x 100 type 1, plain FP32     22: 1.42   26: 1.33   34: 1.35    2.58
 //   20,000 x 100 normal, plain FP32     22: 9.3    26: 9.4    34: 9.9     8.6
-//   40,000 x 31 type 1, plain FP32      15: 0.220             20: 0.217   0.468
+//   50,000 x 28 type 1, plain FP32      15: 0.208             19: 0.187   0.469
 //   20,000 x 31 normal, plain FP32      15: 0.503             20: 0.533   0.503
 //   20,000 x 100 type 1, FP64           32: 1.6    42: 1.37   58: 1.37   12.4
 //   20,000 x 100 normal, FP64                      42: 58     58: 63    101
@@ -353,7 +353,7 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
   }
   // (Objectives of one polytope beyond it go to the register kernel: no type-1 LP of 50,000 does.)
   const bool hands_on = shared && kind == LAZY_SMALL;
-  const bool plain = p->mode == MODE_FP32 && (kind == LAZY_PACK || (q.max_m > q.max_n ? q.max_m : q.max_n) > 64);
+  const bool plain = p->mode == MODE_FP32 && (q.max_m > q.max_n ? q.max_m : q.max_n) > 64;
   const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 || hands_on ? 4 : plain ? 2.5 : 3.25) *
                       (!rpc ? 1 : kind == LAZY_FP64 ? 4 : 2);
   q.kmax = 2 + int(keep * std::sqrt(double(mn)));

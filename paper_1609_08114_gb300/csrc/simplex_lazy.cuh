@@ -444,7 +444,10 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   using Im = Img<T>;
   constexpr int NT = 32 * W, D = NT * R;
   constexpr bool kD = sizeof(T) == 8, SHARED = (KIND & kShared) != 0, PACKED = KIND == kPacked;
-  constexpr int kSpillUnroll = kD ? 1 : RN ? 4 : 2;    // history entries in flight from the workspace
+  // History entries in flight from the workspace (four with one or two warps, or in FP64, take
+  // registers from the rest: 48 x 37 278 us with one, 286 with two; 50,000 x 100 2.04 and 2.08
+  // ms with two and four, FP64 20,000 x 100 1.37 and 1.6 with one and four).
+  constexpr int kSpillUnroll = kD || W == 1 ? 1 : RN ? 4 : 2;
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
   constexpr Im kNone = Im(~Im(0));
   T *hist = reinterpret_cast<T *>(lz_smem + L.hist);
@@ -503,6 +506,8 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   // one polytope (P.shared) are claimed kShareChunk consecutive ones at a time.
   auto claim = [&](int cur) -> int {
     if (!SHARED) return atomicAdd(P.queue, 1);
+    // Another CTA has met a direction of many pivots: no more of them are taken.
+    if (*static_cast<volatile int32_t *>(P.over_count) != 0) return nitems;
     if (cur >= 0 && (cur + 1) % kShareChunk != 0 && cur + 1 < nitems) return cur + 1;
     return atomicAdd(P.queue, 1) * kShareChunk;
   };
@@ -534,11 +539,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   bool again = false;              // the same objective once more, cold
 #pragma unroll 1
   while (item < nitems) {
-    if (tid == 0 && !(SHARED && again)) {
-      nitem = claim(item);
-      // Another CTA has met a direction of many pivots: none after this one here either.
-      if (SHARED && *static_cast<volatile int32_t *>(P.over_count) != 0) nitem = nitems;
-    }
+    if (tid == 0 && !(SHARED && again)) nitem = claim(item);
     again = false;
     // ---- admission: sizes, b >= 0, finite data in the tableau's range ----
     const In *A = static_cast<const In *>(P.B.A) + aoff;
@@ -781,6 +782,8 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
         const Cand<T> col = choose(0, o, nkey, obj, obj, cst);
         if (col.o == kNone) break;
         if (held == (based ? L.kw : L.kmax)) { full = true; break; }
+        // (a start from the wrong basis, and its pivots go to the workspace)
+        if (SHARED && warm && held >= ks && 2 * iters > cold_iters) { full = true; break; }
         const int e = int(col.key) & kIdxMask, cse = col.last;
         // Column e: from A (the slot's tableau) or from the pivot that last stood on it,
         // then the pivots since.
@@ -946,6 +949,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
     }
     if (SHARED && full) {
       if (warm) {                  // the history is full after some warm starts: cold
+        if (2 * iters > cold_iters) cold_left = kShareChunk - 1;
         again = true;
         warm_run = -1;
         continue;
