@@ -327,8 +327,8 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 //   50,000 x 100 type 1, refined        27: 2.25   34: 2.13   37: 2.14    4.19
 //   40,000 x 100 type 1, plain FP32     22: 1.42   26: 1.33   34: 1.35    2.58
 //   20,000 x 100 normal, plain FP32     22: 9.3    26: 9.4    34: 9.9     8.6
-//   50,000 x 28 type 1, plain FP32      15: 0.208             19: 0.187   0.469
-//   20,000 x 31 normal, plain FP32      15: 0.503             20: 0.533   0.503
+//   50,000 x 28 type 1, plain FP32                            19: 0.17    0.46
+//   20,000 x 31 normal, plain FP32                            20: 0.49    0.50
 //   20,000 x 100 type 1, FP64           32: 1.6    42: 1.37   58: 1.37   12.4
 //   20,000 x 100 normal, FP64                      42: 58     58: 63    101
 //   4,000 x 200 x 100 tenth, refined    42: 4.2    72: 5.0   100: 5.4    10.0

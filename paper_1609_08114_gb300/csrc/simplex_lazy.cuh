@@ -269,21 +269,21 @@ __host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warp
 }
 
 // The pivots of the history on the tableau in the slot (`based`; else on A), into the
-// slot: kApplyRows rows of kApplyCols columns (FP64: of one) per thread at a time, with
+// slot: kApplyRows rows of NC columns (kApplyCols; one in FP64 and at 64 registers, where
+// two cost type-1 LPs of 28 x 28 10%) per thread at a time, with
 // every pivot before they are stored, so that one pass over the tableau serves all of
 // them.  Bound by the latency of that pass with a few warps per LP: two columns halve the
 // round trips to L2 (20,000 x 100 x 100 of 126 pivots, plain FP32, inlined: 10.1 ms with one,
 // 9.1 with two, 8.8 with four, which take registers from the kernel).  Not inlined, and
 // called outside of the pivot loop: LPs of few pivots never get here, and its code cost
 // them 4% (50,000 x 100) to 15% (48 x 37) there.
-template <typename T, int NT, bool F64, bool RN>
+template <typename T, int NT, int NC, bool F64, bool RN>
 __device__ __noinline__ void apply_pivots(T *tab, const T *spill, const void *A, int m, int n, int held, bool based,
                                           int hist_at, int ats_at, int ks, int hs, int pn, int ld) {
   extern __shared__ __align__(16) unsigned char lz_smem[];
   __builtin_assume(__isGlobal(tab));
   __builtin_assume(__isGlobal(spill));
   __builtin_assume(__isGlobal(A));
-  constexpr int NC = sizeof(T) == 8 ? 1 : kApplyCols;
   const T *hist = reinterpret_cast<const T *>(lz_smem + hist_at);
   const unsigned *ats = reinterpret_cast<const unsigned *>(lz_smem + ats_at);
   const int nj = (n + NC - 1) / NC, tasks = (m + kApplyRows - 1) / kApplyRows * nj;
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
   // History entries in flight from the workspace (four with one or two warps, or in FP64, take
   // registers from the rest: 48 x 37 278 us with one, 286 with two; 50,000 x 100 2.04 and 2.08
   // ms with two and four, FP64 20,000 x 100 1.37 and 1.6 with one and four).
-  constexpr int kSpillUnroll = kD || W == 1 ? 1 : RN ? 4 : 2;
+  constexpr int kSpillUnroll = kD || (W == 1 && !PACKED) ? 1 : RN && !PACKED ? 4 : 2;
   constexpr unsigned long long kInf = 0x7ff0000000000000ull;
   constexpr Im kNone = Im(~Im(0));
   T *hist = reinterpret_cast<T *>(lz_smem + L.hist);
@@ -939,7 +939,7 @@ __global__ void __launch_bounds__(32 * W, MINB) lazy_kernel(const TableauParams 
       // refinement of an LP whose earlier ones went there.
       const bool refines = !kD && !PACKED && P.mode == MODE_FP32_REFINE && status == LPB_OPTIMAL;
       if (SHARED || (!full && !(refines && based && held > 0))) break;
-      apply_pivots<T, NT, F64, RN>(tableau(), spill, A, m, n, held, based, L.hist, L.at, ks, hs, pn, L.ld);
+      apply_pivots<T, NT, kD || PACKED ? 1 : kApplyCols, F64, RN>(tableau(), spill, A, m, n, held, based, L.hist, L.at, ks, hs, pn, L.ld);
 #pragma unroll
       for (int r = 0; r < R; ++r) rst[r] = cst[r] = -1;
       held = 0;
