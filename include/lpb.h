@@ -173,15 +173,15 @@ lpb_err lpb_destroy(lpb_handle *handle);
  * and these options (depends only on count, max_m, max_n, min_m, min_n,
  * dtype and the options; a solve whose batch declares other sizes than the
  * query may need more and then returns LPB_ENOMEM before any launch).  Part
- * of it holds pivots and tableaux of the automatic kernels, about two matrices A per
- * LP in flight at most under the largest-coefficient rule (20,000 x 100 x 100 in
- * FP64 250 MB, in FP32 75 MB; 150 x 1000 x 1000 3.7 GB, most of it for Phase I),
- * about four in FP64 under the random rule.  A solve, of this or the other calls below,
- * that gets a workspace without room for those, but enough for the kernels that
- * update the whole tableau, runs on these, two to nine times slower: statuses,
- * pivots and bases are the same, and so are FP64 and plain FP32 results; refined
- * ones are as accurate, but not the same bits (objectives of one polytope, which
- * start from one another, end at optima of the same value). */
+ * of it holds pivots and tableaux of the automatic kernels: up to two and a half
+ * matrices A per LP in flight, four under the random rule (20,000 x 100 x 100 in
+ * FP64 370 MB, in FP32 75 MB; 150 x 1000 x 1000 3.7 GB, most of it for Phase I).
+ * A solve, of this or the other calls below, that gets a workspace without room
+ * for those, but enough for the kernels that update the whole tableau, runs on
+ * these, two to nine times slower: statuses, pivots and bases are the same, and
+ * so are FP64 and plain FP32 results; refined ones are as accurate, but not the
+ * same bits (objectives of one polytope, which start from one another, end at
+ * optima of the same value). */
 lpb_err lpb_workspace_size(lpb_handle *handle, const lpb_batch *batch, const lpb_options *opt,
                            size_t *bytes);
 

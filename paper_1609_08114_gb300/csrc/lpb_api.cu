@@ -291,8 +291,8 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // and, with many pivots (normal rows, 70 to 310), everywhere but in plain FP32
 // at 65 to 127 rows or columns with FP64 input, where the warp kernel's tableau in
 // shared memory stays ahead (20,000 LPs or as said, ms before and after):
-//   100, FP64 tableau       101 -> 58     4,000 x 200 x 100       14.9 -> 7.0
-//   64, FP64 tableau       30.7 -> 13.6   64 x 64, FP32 input      6.4 -> 3.2
+//   100, FP64 tableau       101 -> 72     4,000 x 200 x 100       14.9 -> 7.0
+//   64, FP64 tableau       30.7 -> 14.4   64 x 64, FP32 input      6.4 -> 3.2
 //   100, plain FP32         8.6 -> 9.4    64 x 64, plain FP32      2.4 -> 2.3
 // Of the several-LPs-per-warp kernel's passes those of plain FP32 with one or two
 // LPs per warp come here (100,000 LPs: 28 x 28 0.82 -> 0.25, 16 x 31 with FP32
@@ -321,16 +321,21 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // LPs take at most (39 of 50,000 at 100 x 100, 30 at 64 x 64, 22 at 48 x 37, 69 at
 // 300 x 300: about 4 sqrt(min(m, n)); under the random rule two to four times
 // that), which an application would cost more than the chains.  LPs of many pivots
-// would have it earlier, as the entries beyond the shared ones come from L2.  ms with
-// so many kept (normal: normal rows, 126 pivots at 100 x 100; tenth: one entry in ten,
-// 102 pivots at 200 x 100; last: with a full update per pivot):
+// would have it earlier, as the entries beyond the shared ones come from L2.  In FP64
+// the operations count: k pivots cost k^2 (m + n) / 2 in chains -- at 1.5 m n / (m + n)
+// three quarters of the full update's k m n -- and k m n more where they are applied,
+// which LPs that end soon after should not pay.  ms with so many kept (normal: normal
+// rows, 126 pivots at 100 x 100; tenth: one entry in ten, 102 pivots at 200 x 100; last:
+// with a full update per pivot):
 //   50,000 x 100 type 1, refined        27: 2.25   34: 2.13   37: 2.14    4.19
 //   40,000 x 100 type 1, plain FP32     22: 1.42   26: 1.33   34: 1.35    2.58
 //   20,000 x 100 normal, plain FP32     22: 9.3    26: 9.4    34: 9.9     8.6
 //   50,000 x 28 type 1, plain FP32                            19: 0.17    0.46
 //   20,000 x 31 normal, plain FP32                            20: 0.49    0.50
-//   20,000 x 100 type 1, FP64           32: 1.6    42: 1.37   58: 1.37   12.4
-//   20,000 x 100 normal, FP64                      42: 58     58: 63    101
+//   20,000 x 100 type 1, FP64           32: 1.6    42: 1.37   83: 1.37   12.4
+//   20,000 x 100 normal, FP64           42: 58     58: 63     83: 72    101
+//   10,000 x 100 bounded, FP64                     42: 31.8  108: 18.5   51.6
+//   2,000 x 300 type 1, FP64                       71: 5.5   233: 2.7    20.6
 //   4,000 x 200 x 100 tenth, refined    42: 4.2    72: 5.0   100: 5.4    10.0
 //   10,000 x 100 bounded, 64 pivots     42: 9.2    72: 8.2   100: 7.9    17.7
 void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, int shared, Pass *p) {
@@ -354,9 +359,9 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
   // (Objectives of one polytope beyond it go to the register kernel: no type-1 LP of 50,000 does.)
   const bool hands_on = shared && kind == LAZY_SMALL;
   const bool plain = p->mode == MODE_FP32 && (q.max_m > q.max_n ? q.max_m : q.max_n) > 64;
-  const double keep = (kind == LAZY_LARGE ? 7 : kind == LAZY_FP64 || hands_on ? 4 : plain ? 2.5 : 3.25) *
-                      (!rpc ? 1 : kind == LAZY_FP64 ? 4 : 2);
-  q.kmax = 2 + int(keep * std::sqrt(double(mn)));
+  const double keep = kind == LAZY_LARGE ? 7 : hands_on ? 4 : plain ? 2.5 : 3.25;
+  q.kmax = kind == LAZY_FP64 ? 8 + (rpc ? 3 : 1.5) * q.max_m * q.max_n / (q.max_m + q.max_n)
+                             : 2 + (rpc ? 2 : 1) * keep * std::sqrt(double(mn));
   q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL || kind == LAZY_PACK ? 6 + mn / 10 : 8 + mn / 4;
   const int most = 72 * 1024 / ((q.max_m + q.max_n) * eb);      // a third of an SM's shared memory
   if (q.ks > most) q.ks = most;

@@ -27,7 +27,7 @@
 //     that tableau, whenever `ks` more pivots are kept.  The chains then start from the
 //     slot's entries.  The order of operations on an entry is the same, so are the
 //     values.  (20,000 x 100 x 100 with normal rows, 126 pivots: FP64 134 ms when such
-//     LPs started again in the tableau kernel, 58 now, 101 with a full update per pivot;
+//     LPs started again in the tableau kernel, 72 now, 101 with a full update per pivot;
 //     plain FP32 28.9, 9.4 and 8.6.)
 //   * A is read where it lies: one pass over it checks that it is finite (and
 //     leaves it in L2), then a pivot reads the one row and column it needs.
@@ -270,13 +270,13 @@ __host__ __device__ inline LazyLayout lazy_layout(int lim_m, int lim_n, int warp
 
 // The pivots of the history on the tableau in the slot (`based`; else on A), into the
 // slot: kApplyRows rows of NC columns (kApplyCols; one in FP64 and at 64 registers, where
-// two cost type-1 LPs of 28 x 28 10%) per thread at a time, with
-// every pivot before they are stored, so that one pass over the tableau serves all of
-// them.  Bound by the latency of that pass with a few warps per LP: two columns halve the
-// round trips to L2 (20,000 x 100 x 100 of 126 pivots, plain FP32, inlined: 10.1 ms with one,
-// 9.1 with two, 8.8 with four, which take registers from the kernel).  Not inlined, and
-// called outside of the pivot loop: LPs of few pivots never get here, and its code cost
-// them 4% (50,000 x 100) to 15% (48 x 37) there.
+// two cost type-1 LPs of 28 x 28 10%) per thread at a time, with every pivot before they
+// are stored, so that one pass over the tableau serves all of them.  Bound by the latency of
+// that pass with a few warps per LP: two columns halve the round trips to L2 (20,000 x 100 x
+// 100 of 126 pivots, plain FP32, inlined: 10.1 ms with one, 9.1 with two, 8.8 with four,
+// which take registers from the kernel); in FP64 by that pipe.  Not inlined, and called
+// outside of the pivot loop: LPs of few pivots never get here, and its code cost them 4%
+// (50,000 x 100) to 15% (48 x 37) there.
 template <typename T, int NT, int NC, bool F64, bool RN>
 __device__ __noinline__ void apply_pivots(T *tab, const T *spill, const void *A, int m, int n, int held, bool based,
                                           int hist_at, int ats_at, int ks, int hs, int pn, int ld) {
