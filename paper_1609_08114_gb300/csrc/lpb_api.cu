@@ -288,9 +288,9 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 //   30,000 x 48 x 37, FP32 input   1.43 -> 0.29    50,000 x 64    1.46 -> 0.73
 //   50,000 x 100                   4.19 -> 2.03    2,000 x 300    6.0 -> 1.4-1.6
 //   20,000 x 100, FP64 tableau    12.42 -> 1.37
-// and, with many pivots (normal rows, 70 to 310), everywhere but in plain FP32
-// at 65 to 127 rows or columns with FP64 input, where the warp kernel's tableau in
-// shared memory stays ahead (20,000 LPs or as said, ms before and after):
+// and, with many pivots (normal rows, 70 to 310), everywhere but in FP32 at 65 to
+// 127 rows or columns, where the warp kernel's tableau in shared memory stays
+// ahead by 10% plain and 4% refined (20,000 LPs or as said, ms before and after):
 //   100, FP64 tableau       101 -> 72     4,000 x 200 x 100       14.9 -> 7.0
 //   64, FP64 tableau       30.7 -> 14.4   64 x 64, FP32 input      6.4 -> 3.2
 //   100, plain FP32         8.6 -> 9.4    64 x 64, plain FP32      2.4 -> 2.3
@@ -327,7 +327,8 @@ bool warp_auto(const lpb_batch *b, const lpb_options *o, int mode, int lim_m, in
 // which LPs that end soon after should not pay.  ms with so many kept (normal: normal
 // rows, 126 pivots at 100 x 100; tenth: one entry in ten, 102 pivots at 200 x 100; last:
 // with a full update per pivot):
-//   50,000 x 100 type 1, refined        27: 2.25   34: 2.13   37: 2.14    4.19
+//   50,000 x 100 type 1, refined        27: 2.25   34: 2.09   42: 2.03    4.19
+//   20,000 x 100 normal, refined                   34: 42.5   42: 43.1   40.7
 //   40,000 x 100 type 1, plain FP32     22: 1.42   26: 1.33   34: 1.35    2.58
 //   20,000 x 100 normal, plain FP32     22: 9.3    26: 9.4    34: 9.9     8.6
 //   50,000 x 28 type 1, plain FP32                            19: 0.17    0.46
@@ -358,8 +359,10 @@ void lazy_pass(const DeviceInfo &d, const lpb_batch *b, const lpb_options *o, in
   }
   // (Objectives of one polytope beyond it go to the register kernel: no type-1 LP of 50,000 does.)
   const bool hands_on = shared && kind == LAZY_SMALL;
-  const bool plain = p->mode == MODE_FP32 && (q.max_m > q.max_n ? q.max_m : q.max_n) > 64;
-  const double keep = kind == LAZY_LARGE ? 7 : hands_on ? 4 : plain ? 2.5 : 3.25;
+  // (After the warp kernel's refined passes the FP64 re-solve dwarfs what an LP of many
+  // pivots takes here.)
+  const bool two = (q.max_m > q.max_n ? q.max_m : q.max_n) > 64;       // two warps per LP
+  const double keep = kind == LAZY_LARGE ? 7 : hands_on ? 4 : two && p->mode == MODE_FP32 ? 2.5 : two && p->warp ? 4 : 3.25;
   q.kmax = kind == LAZY_FP64 ? 8 + (rpc ? 3 : 1.5) * q.max_m * q.max_n / (q.max_m + q.max_n)
                              : 2 + (rpc ? 2 : 1) * keep * std::sqrt(double(mn));
   q.ks = kind == LAZY_FP64 ? 4 + mn / 25 : rpc ? 6 + mn / 2 : kind == LAZY_SMALL || kind == LAZY_PACK ? 6 + mn / 10 : 8 + mn / 4;
